@@ -430,7 +430,8 @@ pmf_status pmf_chain_set_warps(pmf_system *sys, int chain, int warps);
  * replica, every replica's steps in one launch per 1e5-step chunk.
  * ctas >= 0: persistent launch of min(ctas, replicas) CTAs (ctas = 0: every
  * CTA slot the GPU holds at once) that take work items of seg_steps steps
- * (0: 1000) of one replica from a device queue, in segment-major order
+ * (0: 1000, or an eighth of the launch, at least 16, where that is less and the
+ * replicas do not all fit at once) of one replica from a device queue, in segment-major order
  * (ctas = 0 picks: every slot if the replicas fill them, else a whole number
  * of CTAs per SM when that is at least 3, else one CTA per replica); a
  * replica's next segment waits (at most 60 s, then PMF_ETIMEOUT) until its

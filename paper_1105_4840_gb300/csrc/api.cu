@@ -1929,7 +1929,7 @@ pmf_status pmf_chain_autotune(pmf_system *sys, const double *lambda, int n_windo
     if (pmf_status s = pmf_run_prepare(sys, lambda, n_windows, &q, &run)) return s;
     std::unique_ptr<pmf_run, void (*)(pmf_run *)> guard(run, pmf_destroy_run);
     int best = m.warps(), best_grid = m.grid_ctas();
-    const int seg = m.seg_steps();
+    const int seg = m.seg_request();
     double best_t = 1e300;
     GpuTimer timer;
     // launch shapes: the automatic persistent grid, and one persistent CTA

@@ -1204,6 +1204,7 @@ struct ChainModel::Impl {
     int variant = 0;         // cost model of the FP32 schedule (kSchedWeights)
     int grid_ctas = 0;       // persistent CTAs: 0 = auto, < 0 = one CTA per replica
     int seg_steps = 1000;    // steps per persistent work item
+    bool seg_auto = true;    //   (the default: shorter in short launches, see auto_segment)
     // schedules of the packed batch launch, per team size (warps per replica)
     struct TeamSched {
         int4 *units = nullptr;
@@ -1251,11 +1252,13 @@ cudaError_t ChainModel::set_grid(int ctas, int seg_steps)
     if (seg_steps < 0) return cudaErrorInvalidValue;
     p->grid_ctas = ctas;
     p->seg_steps = seg_steps > 0 ? seg_steps : 1000;
+    p->seg_auto = seg_steps == 0;
     ++p->generation;
     return cudaSuccess;
 }
 int ChainModel::grid_ctas() const { return p->grid_ctas; }
 int ChainModel::seg_steps() const { return p->seg_steps; }
+int ChainModel::seg_request() const { return p->seg_auto ? 0 : p->seg_steps; }
 unsigned ChainModel::generation() const { return p->generation; }
 
 cudaError_t ChainModel::set_warps(int NW)
@@ -1377,6 +1380,20 @@ static ChainArgs<R> fill_args(const ChainModel::Impl *m, const ChainDevice<R> &d
     return a;
 }
 
+// Steps of a work item when the caller left the default and the replicas do
+// not all fit at once: an eighth of the launch, 16 to 1000.  With the fixed
+// 1000 a launch shorter than that could not migrate, and 672 replicas of the
+// 104-bead chain on 608 CTA slots ran as two waves (400 steps: 3.44 ms; in
+// two, four, eight, sixteen segments 2.89, 2.64, 2.66, 2.76 ms, each segment
+// costing about two steps of loading, storing and one more force evaluation;
+// 336 replicas of 201 beads on 304 slots, 200 steps: 3.23, 2.79, 2.72, 2.64,
+// 2.80 ms).  From 8000 steps on the item is 1000 steps as before.
+static int auto_segment(long long steps)
+{
+    const long long s = (steps + 7) / 8;
+    return (int)(s < 16 ? 16 : (s > 1000 ? 1000 : s));
+}
+
 template <typename R, int NW>
 static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, const RunLaunch &L, cudaStream_t st)
 {
@@ -1423,6 +1440,7 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
             want = L.n_blocks >= slots ? slots : (per_sm >= 3 ? per_sm * sms : L.n_blocks);
         }
         grid = (int)std::min<long long>(want, L.n_blocks);
+        if (!L.sequential && m->seg_auto && grid < L.n_blocks) a.seg_steps = auto_segment(L.step_end - L.step_begin);
         const long long nseg = L.sequential ? (L.step_end / L.window_steps) * a.subs_per_window
                                             : (L.step_end - L.step_begin + a.seg_steps - 1) / a.seg_steps;
         a.persistent = 1;

@@ -104,10 +104,12 @@ public:
     unsigned generation() const;
     // Launch shape: ctas > 0 persistent with that many CTAs, 0 persistent
     // with every CTA slot of the GPU, < 0 one CTA per replica; seg_steps =
-    // steps per persistent work item (0: 1000).  Bumps the generation.
+    // steps per persistent work item (0: 1000, less in short launches).
+    // Bumps the generation.
     cudaError_t set_grid(int ctas, int seg_steps);
     int grid_ctas() const;
     int seg_steps() const;
+    int seg_request() const;  // as set: 0 while the default is left
     // FP32 packed batch launch: the schedule of team size G (cached on the
     // device) and the shared memory of one replica team of that size
     cudaError_t team_schedule(int G, const int4 **units, const int **count, int *max_units);
