@@ -40,8 +40,8 @@ template <typename R> struct alignas(2 * sizeof(R)) Vec2 {
 };
 
 template <typename R> struct ChainArgs {
-    const Vec4<R> *bead_pos0;  // [Np] start state, w = sigma/2; pads far away
-    const Vec2<R> *bead_eq;    // [Np] (sqrt(24 eps), q sqrt(ke)); zero for pads
+    const Vec4<R> *bead_pos0;  // [Np] start state, w = kLjScale sigma/2; pads far away
+    const Vec2<R> *bead_eq;    // [Np] (sqrt(12 eps), q sqrt(ke)); zero for pads
     const R *bead_invm;        // [Np] 1/m, 0 for pads
     const Vec4<R> *dih;        // [N] (K1 cos d1, K2 cos d2, K3 cos d3, nonzero)
     Vec4<R> *state;            // [n_rep][2][Np] positions, velocities
@@ -197,9 +197,9 @@ __device__ __forceinline__ R pair_fr(const Vec4<R> &pi, const Vec2<R> &qi, const
     const R ri2 = ri * ri;
     const R sg = pi.w + pj.w;
     const R x2 = sg * sg * ri2;
-    const R x6 = x2 * x2 * x2;
-    const R lj = (qi.x * qj.x) * x6 * (R(2) * x6 - R(1));  // 24 eps_ij (2 x^12 - x^6)
-    return ((qi.y * qj.y) * ri + lj) * ri2;                 // -dU/dr / r
+    const R z = x2 * x2 * x2;                 // 2 (s_ij / r)^6
+    const R g = (qi.x * qj.x) * z;            // 12 eps_ij z; the LJ part is g (z - 1)
+    return (g * z + ((qi.y * qj.y) * ri - g)) * ri2;  // -dU/dr / r
 }
 
 template <typename R, int KIND, bool DUAL>
@@ -280,6 +280,11 @@ __device__ __forceinline__ void ring_piece(const Smem<R> &s, Vec4<R> *fw, int I1
 }
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+// a b + c and a b - c on the two halves as scalar FFMAs: a packed FFMA2 with
+// three distinct operand pairs reads six registers and takes 3.16 cycles of
+// the FP32 pipe (one warp per scheduler, dependent chains of eight), two
+// scalar FFMAs 2.18, and their sign modifiers are free.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return f2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)); }
 
 // Quad pieces (FP32): lane l holds two neighbouring i-beads of its ring,
 // i1 at ring index l and i2 at l + 1, and at ring step t meets the j-beads at
@@ -290,27 +295,36 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 // one rotation (by two lanes) of the j-force streams, halving the shared
 // loads and shuffles per pair; the two i-beads form the packed f32x2 operand.
 //
+// The Lennard-Jones part is g z - g with z = 2 (s_ij / r)^6 and g = 12 eps_ij z
+// (the factors 2^(1/6) and 12 sit in the stored parameters), folded into the
+// Coulomb term as (q ri - g) + g z: 24 FP32 operations a pair where
+// 24 eps (2 x^12 - x^6) takes 25.  The steps are one straight line: the masks
+// are selects, not branches, every i-tile is full (I < J, and a W 32 diagonal
+// is), and each tile is flushed by one read-modify-write, so the compiler can
+// overlap the steps.  What bounds a piece is the number of registers for that
+// overlap: alone on its scheduler a warp takes about 230 cycles per ring step
+// with 128 registers, 300 with 96, against 100 of FP32 pipe; SCALAR (both FMAs
+// of the pair as scalar FFMAs) is the faster form with 128 registers and
+// spills with 96.  Same results in both forms.  One CTA per SM, 4 warps:
+// 104 beads 7890 -> 7170 cycles a step, 333 beads 41150 -> 31480; 672 replicas
+// of 104 beads 100.4 -> 107.0 M replica-steps/s (1000 steps).
+//
 // SPLIT pieces jump from ring step TB + 6 to TB + 16 halfway (offsets 0..15
 // then 16..31 of an off-diagonal W 32 ring in one piece): the j-force streams
 // then rotate by ten lanes once instead of two.
-template <int W, int NST, bool SPLIT>
-__device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw, int I, int J, int TB, bool diag,
-                                           bool near, int wI, int lane)
+template <int W, int NST, int TB, bool DIAG, bool SPLIT, bool SCALAR>
+__device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw, int I, int J, int lane)
 {
     constexpr int D = pair_offset(W);
     const int lr = lane & (W - 1);
     const int l2 = (lane & ~(W - 1)) | ((lr + 1) & (W - 1));  // lane of i2 within the i-tile
-    const bool on1 = lane < wI, on2 = l2 < wI;
-    Vec4<float> p1{-1e4f, -1e4f, -1e4f, 0.f}, p2{-2e4f, -1e4f, -1e4f, 0.f};
-    Vec2<float> q1{0.f, 0.f}, q2{0.f, 0.f};
-    if (on1) { p1 = s.posd[I * 64 + lane]; q1 = s.eqd[I * 64 + lane]; }
-    if (on2) { p2 = s.posd[I * 64 + l2]; q2 = s.eqd[I * 64 + l2]; }
+    const Vec4<float> p1 = s.posd[I * 64 + lane], p2 = s.posd[I * 64 + l2];
+    const Vec2<float> q1 = s.eqd[I * 64 + lane], q2 = s.eqd[I * 64 + l2];
     // i-bead data duplicated across the packed halves (streams a, b)
     const float2 nx1 = f2(-p1.x, -p1.x), ny1 = f2(-p1.y, -p1.y), nz1 = f2(-p1.z, -p1.z);
     const float2 nx2 = f2(-p2.x, -p2.x), ny2 = f2(-p2.y, -p2.y), nz2 = f2(-p2.z, -p2.z);
     const float2 s1 = f2(p1.w, p1.w), s2 = f2(p2.w, p2.w);
     const float2 e1 = f2(q1.x, q1.x), e2 = f2(q2.x, q2.x), c1 = f2(q1.y, q1.y), c2 = f2(q2.y, q2.y);
-    const float2 two = f2(2.f, 2.f), mone = f2(-1.f, -1.f);
     float2 f1x = f2(0.f, 0.f), f1y = f1x, f1z = f1x, f2x = f1x, f2y = f1x, f2z = f1x;
     float2 fjx = f1x, fjy = f1x, fjz = f1x;
     const float4 *PA = s.posa + 64 * J + lr, *PB = s.posb + 64 * J + lr;
@@ -318,8 +332,7 @@ __device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw
     const int src = (lane & ~(W - 1)) | ((lr + 2) & (W - 1));
     const int src_jump = (lane & ~(W - 1)) | ((lr + 10) & (W - 1));
     const int gi1 = I * 32 + lane, gi2 = I * 32 + l2;
-    const bool mask_near = near && TB < 4;
-    const bool mask_half = diag && lr >= (W >> 1);
+    const bool mask_half = DIAG && lr >= (W >> 1);
 #pragma unroll
     for (int k = 0; k < NST; ++k) {
         const int t = TB + 2 * k + ((SPLIT && 2 * k >= NST) ? 8 : 0);
@@ -337,16 +350,17 @@ __device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw
         const float2 iq1 = __fmul2_rn(ri1, ri1), iq2 = __fmul2_rn(ri2_, ri2_);
         const float2 sg1 = __fadd2_rn(s1, sj), sg2 = __fadd2_rn(s2, sj);
         const float2 x21 = __fmul2_rn(__fmul2_rn(sg1, sg1), iq1), x22 = __fmul2_rn(__fmul2_rn(sg2, sg2), iq2);
-        const float2 x61 = __fmul2_rn(__fmul2_rn(x21, x21), x21), x62 = __fmul2_rn(__fmul2_rn(x22, x22), x22);
-        const float2 lj1 = __fmul2_rn(__fmul2_rn(__fmul2_rn(e1, ej), x61), __ffma2_rn(x61, two, mone));
-        const float2 lj2 = __fmul2_rn(__fmul2_rn(__fmul2_rn(e2, ej), x62), __ffma2_rn(x62, two, mone));
-        float2 fr1 = __fmul2_rn(__ffma2_rn(__fmul2_rn(c1, cj), ri1, lj1), iq1);
-        float2 fr2 = __fmul2_rn(__ffma2_rn(__fmul2_rn(c2, cj), ri2_, lj2), iq2);
-        if (mask_near && t < 4) {  // exclusions |i - j| <= 2 can only meet stream a at ring offsets <= 2
+        const float2 z1 = __fmul2_rn(__fmul2_rn(x21, x21), x21), z2 = __fmul2_rn(__fmul2_rn(x22, x22), x22);
+        const float2 g1 = __fmul2_rn(__fmul2_rn(e1, ej), z1), g2 = __fmul2_rn(__fmul2_rn(e2, ej), z2);
+        const float2 h1 = __fmul2_rn(c1, cj), h2 = __fmul2_rn(c2, cj);
+        const float2 u1 = fma2(h1, ri1, f2(-g1.x, -g1.y)), u2 = fma2(h2, ri2_, f2(-g2.x, -g2.y));
+        float2 fr1 = __fmul2_rn(SCALAR ? fma2(g1, z1, u1) : __ffma2_rn(g1, z1, u1), iq1);
+        float2 fr2 = __fmul2_rn(SCALAR ? fma2(g2, z2, u2) : __ffma2_rn(g2, z2, u2), iq2);
+        if (t < 4) {  // exclusions |i - j| <= 2 can only meet stream a at ring offsets <= 2
             const int gj = J * 32 + ((lr + t) & (W - 1));
-            const int d1 = gi1 - gj, d2 = gi2 - gj;
-            if (d1 <= 2 && d1 >= -2) fr1.x = 0.f;
-            if (d2 <= 2 && d2 >= -2) fr2.x = 0.f;
+            const unsigned d1 = (unsigned)(gi1 - gj + 2), d2 = (unsigned)(gi2 - gj + 2);
+            fr1.x = d1 <= 4u ? 0.f : fr1.x;
+            fr2.x = d2 <= 4u ? 0.f : fr2.x;
         }
         if (mask_half && k == NST - 1) fr1.y = 0.f;  // offset W/2 of a diagonal: counted from one side only
         f1x = __ffma2_rn(fr1, dx1, f1x); f1y = __ffma2_rn(fr1, dy1, f1y); f1z = __ffma2_rn(fr1, dz1, f1z);
@@ -363,15 +377,17 @@ __device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw
             fjz.y = __shfl_sync(0xffffffffu, fjz.y, sl);
         }
     }
-    if (on1) {
+    // flush: one read-modify-write per tile; the other half of a bead's sum
+    // (i2 of the lane before, stream b of the lane D before) comes by shuffle
+    {
+        const int from = (lane & ~(W - 1)) | ((lr - 1) & (W - 1));  // its i2 is this lane's i1
+        const float gx = __shfl_sync(0xffffffffu, f2x.x + f2x.y, from);
+        const float gy = __shfl_sync(0xffffffffu, f2y.x + f2y.y, from);
+        const float gz = __shfl_sync(0xffffffffu, f2z.x + f2z.y, from);
         Vec4<float> f = fw[I * 32 + lane];
         f.x -= f1x.x + f1x.y; f.y -= f1y.x + f1y.y; f.z -= f1z.x + f1z.y;
+        f.x -= gx; f.y -= gy; f.z -= gz;
         fw[I * 32 + lane] = f;
-    }
-    if (on2) {  // l2 is a permutation of the lanes: distinct beads within this pass
-        Vec4<float> f = fw[I * 32 + l2];
-        f.x -= f2x.x + f2x.y; f.y -= f2y.x + f2y.y; f.z -= f2z.x + f2z.y;
-        fw[I * 32 + l2] = f;
     }
 #pragma unroll
     for (int o = W; o < 32; o <<= 1) {
@@ -379,17 +395,20 @@ __device__ __forceinline__ void quad_piece(const Smem<float> &s, Vec4<float> *fw
         fjy.x += __shfl_xor_sync(0xffffffffu, fjy.x, o); fjy.y += __shfl_xor_sync(0xffffffffu, fjy.y, o);
         fjz.x += __shfl_xor_sync(0xffffffffu, fjz.x, o); fjz.y += __shfl_xor_sync(0xffffffffu, fjz.y, o);
     }
-    if (lane < W) {
-        const int tl = TB + 2 * (NST - 1) + (SPLIT ? 8 : 0);
-        const int ba = J * 32 + ((lr + tl) & (W - 1));
-        Vec4<float> f = fw[ba];
+    const int from_b = (lane & ~(W - 1)) | ((lr - D) & (W - 1));
+    fjx.y = __shfl_sync(0xffffffffu, fjx.y, from_b);
+    fjy.y = __shfl_sync(0xffffffffu, fjy.y, from_b);
+    fjz.y = __shfl_sync(0xffffffffu, fjz.y, from_b);
+    __syncwarp();
+    if (W == 32 || lane < W) {
+        constexpr int tl = TB + 2 * (NST - 1) + (SPLIT ? 8 : 0);
+        const int bj = J * 32 + ((lr + tl) & (W - 1));
+        Vec4<float> f = fw[bj];
         f.x += fjx.x; f.y += fjy.x; f.z += fjz.x;
-        fw[ba] = f;
-        const int bb = J * 32 + ((lr + tl + D) & (W - 1));
-        f = fw[bb];
         f.x += fjx.y; f.y += fjy.y; f.z += fjz.y;
-        fw[bb] = f;
+        fw[bj] = f;
     }
+    __syncwarp();
 }
 
 // Diagonal of a ragged last tile (width 8 or 16), scalar, ring steps 1..W/2;
@@ -447,16 +466,16 @@ __device__ __noinline__ void ragged_diag_piece(const Smem<float> &s, Vec4<float>
 //   23: W 32 diagonal, t = 2, 4, 6, 8 (+8)
 //   24: W 16, t = 1, 3, 5, 7 (+8)       25: W 8, t = 1, 3 (+4)
 //   8, 10: diagonal of a ragged tile of width 16 / 8, scalar
-__device__ __forceinline__ void run_packed_piece(const Smem<float> &s, Vec4<float> *fw, int kind, int I, int J,
-                                                 bool near, int wI, int lane)
+template <bool SCALAR>
+__device__ __forceinline__ void run_packed_piece(const Smem<float> &s, Vec4<float> *fw, int kind, int I, int J, int lane)
 {
     switch (kind) {
-    case 21: quad_piece<32, 4, false>(s, fw, I, J, 1, false, near, wI, lane); break;
-    case 22: quad_piece<32, 4, false>(s, fw, I, J, 17, false, near, wI, lane); break;
-    case 23: quad_piece<32, 4, false>(s, fw, I, J, 2, true, near, wI, lane); break;
-    case 24: quad_piece<16, 4, false>(s, fw, I, J, 1, false, near, wI, lane); break;
-    case 26: quad_piece<32, 8, true>(s, fw, I, J, 1, false, near, wI, lane); break;
-    case 25: quad_piece<8, 2, false>(s, fw, I, J, 1, false, near, wI, lane); break;
+    case 21: quad_piece<32, 4, 1, false, false, SCALAR>(s, fw, I, J, lane); break;
+    case 22: quad_piece<32, 4, 17, false, false, SCALAR>(s, fw, I, J, lane); break;
+    case 23: quad_piece<32, 4, 2, true, false, SCALAR>(s, fw, I, J, lane); break;
+    case 24: quad_piece<16, 4, 1, false, false, SCALAR>(s, fw, I, J, lane); break;
+    case 26: quad_piece<32, 8, 1, false, true, SCALAR>(s, fw, I, J, lane); break;
+    case 25: quad_piece<8, 2, 1, false, false, SCALAR>(s, fw, I, J, lane); break;
     case 8: ragged_diag_piece(s, fw, J, 16, lane); break;
     case 10: ragged_diag_piece(s, fw, J, 8, lane); break;
     default: break;  // the host schedule emits only the kinds above
@@ -617,7 +636,7 @@ struct Team {
     }
 };
 
-template <typename R, int NW, bool SMD>
+template <typename R, int NW, bool SMD, bool SCALAR>
 __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R> &s, R lam, long long done,
                                             long long nequil, long long sample_base, bool first, uint32_t uid,
                                             long long rec, const Team &tm)
@@ -653,14 +672,21 @@ __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R>
         Vec4<R> *fw_mine = s.fw + warp * a.Np;
         const int cnt = s.ucount[warp];
         const int4 *u = s.units + warp * a.max_units;
-        for (int q = 0; q < cnt; ++q) {
-            const int4 e = u[q];  // (I1, I2 or -1, J, kind | near1 << 8 | near2 << 9)
-            const int kind = e.w & 0xff;
-            const bool n1 = (e.w >> 8) & 1, n2 = (e.w >> 9) & 1;
-            const int wI = tile_width(e.x, a.n_tiles, a.w_last);
-            if constexpr (kPacked<R>) {
-                run_packed_piece(s, fw_mine, kind, e.x, e.z, n1, wI, lane);
-            } else {
+        if constexpr (kPacked<R>) {
+            // (kind | I << 8 | J << 16, in x); the next piece's word is on its
+            // way while this piece runs
+            int next = cnt > 0 ? u[0].x : 0;
+            for (int q = 0; q < cnt; ++q) {
+                const int e = next;
+                if (q + 1 < cnt) next = u[q + 1].x;
+                run_packed_piece<SCALAR>(s, fw_mine, e & 0xff, (e >> 8) & 0xff, e >> 16, lane);
+            }
+        } else {
+            for (int q = 0; q < cnt; ++q) {
+                const int4 e = u[q];  // (I1, I2 or -1, J, kind | near1 << 8 | near2 << 9)
+                const int kind = e.w & 0xff;
+                const bool n1 = (e.w >> 8) & 1, n2 = (e.w >> 9) & 1;
+                const int wI = tile_width(e.x, a.n_tiles, a.w_last);
                 if (e.y >= 0) run_piece<R, true>(s, fw_mine, kind, e.x, e.y, e.z, n1, n2, wI, lane);
                 else run_piece<R, false>(s, fw_mine, kind, e.x, 0, e.z, n1, false, wI, lane);
             }
@@ -690,7 +716,7 @@ template <> __device__ __forceinline__ Vec4<double> load_cg<double>(const Vec4<d
 // state record, and goes back to it at the end, so a replica's trajectory
 // does not depend on how its steps are cut into launches or segments.
 // Returns false when the run was aborted (non-finite state).
-template <typename R, int NW, bool SMD>
+template <typename R, int NW, bool SMD, bool SCALAR>
 __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s, int rep, int w, int r,
                                          long long s0, long long s1, long long origin, const Team &tm)
 {
@@ -756,9 +782,6 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
     }
     const long long nequil = origin + a.nequil_w[w];  // equilibration counts from the window's first step
     const long long sample_base = a.off_w[w] + (long long)r * a.tw[w];
-    force_phase<R, NW, SMD>(a, s, SMD ? (R)smd_lambda(a.lambda[0], a.smd_vdt, s0, nequil) : lam, s0, nequil,
-                            sample_base, true, uid, -1, tm);
-    tm.sync();
     // record q is taken after nequil + (q + 1) stride steps: the first one
     // after s0 and the step it falls on (one division per segment instead
     // of a 64-bit remainder per step)
@@ -766,7 +789,21 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
     long long rec_step = nequil + (rec_q + 1) * a.stride;
 
     const int warp = tid >> 5, lane = tid & 31;
+    // one call site of force_phase for the segment's first evaluation and all
+    // later ones: the pieces' unrolled code exists once per kernel
     for (long long step = s0;; ++step) {
+        long long rec = -1;
+        if (step == rec_step) {
+            rec = rec_q++;
+            rec_step += a.stride;
+        }
+        force_phase<R, NW, SMD, SCALAR>(a, s, SMD ? (R)smd_lambda(a.lambda[0], a.smd_vdt, step, nequil) : lam, step, nequil,
+                                sample_base, step == s0, uid, rec, tm);
+        tm.sync();
+        if (step > s0 && *s.flag) {
+            if (tid == 0) atomicOr(a.err, kErrNonFinite);
+            return false;
+        }
         // one warp per 32-bead tile (warp-uniform loop: the packed copy is
         // rebuilt with shuffles by the whole warp)
         for (int tile = warp; tile < a.n_tiles; tile += NW) {
@@ -794,7 +831,7 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
                 Vec4<R> v = s.vel[b];
                 if (step > s0) { v.x += hdt * F.x * im; v.y += hdt * F.y * im; v.z += hdt * F.z * im; }
                 if (step < s1) {
-                    const Vec4<R> p4 = s.posd[(b >> 5) * 64 + (b & 31)];  // position and sigma/2
+                    const Vec4<R> p4 = s.posd[(b >> 5) * 64 + (b & 31)];  // position and half width
                     V3<R> p{p4.x, p4.y, p4.z};
                     v.x += hdt * F.x * im; v.y += hdt * F.y * im; v.z += hdt * F.z * im;
                     p.x += hdt * v.x; p.y += hdt * v.y; p.z += hdt * v.z;
@@ -823,18 +860,6 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
                          (NW - a.n_tiles) * 32);
         if (step >= s1) break;
         tm.sync();
-        long long rec = -1;
-        if (step + 1 == rec_step) {
-            rec = rec_q++;
-            rec_step += a.stride;
-        }
-        force_phase<R, NW, SMD>(a, s, SMD ? (R)smd_lambda(a.lambda[0], a.smd_vdt, step + 1, nequil) : lam,
-                                step + 1, nequil, sample_base, false, uid, rec, tm);
-        tm.sync();
-        if (*s.flag) {
-            if (tid == 0) atomicOr(a.err, kErrNonFinite);
-            return false;
-        }
     }
     tm.sync();
     for (int b = tid; b < a.Np; b += NW * 32) {
@@ -927,9 +952,8 @@ __device__ __forceinline__ Smem<R> carve_smem(unsigned char *p, const ChainArgs<
     return s;
 }
 
-template <typename R, int NW, bool SMD>
-__global__ void __launch_bounds__(NW * 32, sizeof(R) == 4 ? (NW == 4 ? 5 : (NW == 5 ? 4 : (NW == 6 ? 3 : 2))) : 1)
-    chain_kernel(const ChainArgs<R> a)
+template <typename R, int NW, int CTAS, bool SMD>
+__global__ void __launch_bounds__(NW * 32, CTAS) chain_kernel(const ChainArgs<R> a)
 // SMD: the constant-velocity pulling variant (a separate instantiation, so
 // the window runs carry none of its per-step work bookkeeping).
 // FP32 with 4 warps: five CTAs per SM fit; 6 and 8 warps trade occupancy for
@@ -994,7 +1018,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(R) == 4 ? (NW == 4 ? 5 : (NW =
             s1 = s1 < nsteps ? s1 : nsteps;
         }
         const Team tm{(int)threadIdx.x, 0, NW * 32};
-        if ((s0 < s1 || a.force_out != nullptr) && !simulate<R, NW, SMD>(a, s, rep, w, r, s0, s1, origin, tm)) return;
+        if ((s0 < s1 || a.force_out != nullptr) && !simulate<R, NW, SMD, NW == 4 && CTAS == 4>(a, s, rep, w, r, s0, s1, origin, tm)) return;
         if (a.persistent) {
             __syncthreads();  // the replica's state record is written
             if (threadIdx.x == 0) {
@@ -1137,6 +1161,13 @@ template <typename R> size_t chain_smem_bytes(const ChainGeometry &g, int NW, in
     return fit ? b + x : b;
 }
 
+// A schedule record as the kernels read it.
+static int4 device_unit(const UnitDesc &u, bool packed)
+{
+    if (packed) return int4{u.kind | (u.I1 << 8) | (u.J << 16), 0, 0, 0};
+    return int4{u.I1, u.I2, u.J, u.kind | (u.near1 << 8) | (u.near2 << 9)};
+}
+
 // Device copy of one chain in precision R.
 template <typename R> struct ChainDevice {
     Vec4<R> *pos0 = nullptr;
@@ -1145,6 +1176,10 @@ template <typename R> struct ChainDevice {
     Vec4<R> *dih = nullptr;
 };
 
+// 2^(1/6): half widths are stored times this, so that (s_i + s_j)^6 / r^6 is
+// z = 2 (s_ij / r)^6 and -dU_LJ/dr r = 12 eps_ij (z^2 - z).
+constexpr double kLjScale = 1.122462048309372981433533;
+
 template <typename R> static cudaError_t upload_chain(const ChainHost &h, const ChainGeometry &g, ChainDevice<R> &d)
 {
     std::vector<Vec4<R>> pos(g.Np), dih(g.N);
@@ -1152,8 +1187,8 @@ template <typename R> static cudaError_t upload_chain(const ChainHost &h, const 
     std::vector<R> invm(g.Np, R(0));
     for (int b = 0; b < g.Np; ++b) {
         if (b < g.N) {
-            pos[b] = Vec4<R>{(R)h.pos0[3 * b], (R)h.pos0[3 * b + 1], (R)h.pos0[3 * b + 2], (R)(0.5 * h.sigma[b])};
-            eq[b] = Vec2<R>{(R)std::sqrt(24.0 * h.epsilon[b]), (R)(h.charge[b] * std::sqrt(h.coulomb_k))};
+            pos[b] = Vec4<R>{(R)h.pos0[3 * b], (R)h.pos0[3 * b + 1], (R)h.pos0[3 * b + 2], (R)(kLjScale * 0.5 * h.sigma[b])};
+            eq[b] = Vec2<R>{(R)std::sqrt(12.0 * h.epsilon[b]), (R)(h.charge[b] * std::sqrt(h.coulomb_k))};
             invm[b] = (R)(1.0 / h.mass[b]);
         } else {  // pads: distinct far positions, no interaction
             pos[b] = Vec4<R>{(R)(1.0e4 + 100.0 * b), (R)1.0e4, (R)1.0e4, R(0)};
@@ -1282,7 +1317,7 @@ cudaError_t ChainModel::set_warps(int NW)
         for (size_t q = 0; q < sched[w].size(); ++q) {
             const UnitDesc &u = sched[w][q];
             flat[(size_t)w * mx + q] =
-                int4{u.I1, u.I2, u.J, u.kind | (u.near1 << 8) | (u.near2 << 9)};
+                device_unit(u, p->precision != 1);
         }
     }
     p->max_units = mx;
@@ -1394,7 +1429,7 @@ static int auto_segment(long long steps)
     return (int)(s < 16 ? 16 : (s > 1000 ? 1000 : s));
 }
 
-template <typename R, int NW>
+template <typename R, int NW, int CTAS>
 static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, const RunLaunch &L, cudaStream_t st)
 {
     if (L.smd_vdt != 0.0 && L.wout == nullptr) return cudaErrorInvalidValue;  // a pulled run records its work
@@ -1402,7 +1437,7 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
     bool extras = false;
     const size_t smem = chain_smem_bytes<R>(m->geo, NW, m->max_units, &extras);
     a.static_in_smem = extras ? 1 : 0;
-    void (*kern)(const ChainArgs<R>) = a.smd ? chain_kernel<R, NW, true> : chain_kernel<R, NW, false>;
+    void (*kern)(const ChainArgs<R>) = a.smd ? chain_kernel<R, NW, CTAS, true> : chain_kernel<R, NW, CTAS, false>;
     // The attribute is the kernel's upper limit, shared by every chain that
     // launches it: raise it to the device's opt-in maximum rather than to this
     // chain's size, so launches captured earlier in a graph (other chains,
@@ -1518,7 +1553,7 @@ __device__ __forceinline__ bool pack_team(const ChainArgs<R> &a, unsigned char *
 {
     unsigned char *tail = nullptr;
     const Smem<R> s = carve_smem<R, G>(base, a, &tail);
-    return simulate<R, G, false>(a, s, rep, rep / a.replicas, rep % a.replicas, s0, s1, 0, tm);
+    return simulate<R, G, false, false>(a, s, rep, rep / a.replicas, rep % a.replicas, s0, s1, 0, tm);
 }
 
 template <typename R>
@@ -1592,7 +1627,7 @@ cudaError_t ChainModel::team_schedule(int G, const int4 **units, const int **cou
             cnt[w] = (int)sched[w].size();
             for (size_t q = 0; q < sched[w].size(); ++q) {
                 const UnitDesc &u = sched[w][q];
-                flat[(size_t)w * mx + q] = int4{u.I1, u.I2, u.J, u.kind | (u.near1 << 8) | (u.near2 << 9)};
+                flat[(size_t)w * mx + q] = device_unit(u, true);
             }
         }
         cudaError_t e;
@@ -1756,13 +1791,31 @@ int pack_plan_packs(const PackPlan *plan) { return plan ? plan->args.n_packs : 0
 int pack_plan_grid(const PackPlan *plan) { return plan ? plan->grid : 0; }
 size_t pack_plan_smem(const PackPlan *plan) { return plan ? plan->smem : 0; }
 
+// Four warps a replica, two builds of the same arithmetic (bit-identical):
+// four CTAs per SM with 128 registers a thread, which lets the compiler
+// overlap the ring steps, or five with 96.  The fifth CTA pays only where
+// there are replicas for it and the pair work is short: cycles per step with
+// 1344 replicas, four / five CTAs: 24 beads 6698 / 6413, 40 10928 / 9925,
+// 64 11533 / 11371, 72 17455 / 16577, 80 19498 / 19970, 104 24999 / 25923;
+// with 672 replicas four win at every length (40 beads 5739 / 5997, 104
+// 12997 / 13863).
+static bool small_chain_ctas(const ChainGeometry &g, int n_rep)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return false;
+    return g.Np <= 72 && n_rep >= 5 * sms;
+}
+
 cudaError_t ChainModel::launch(const RunLaunch &L, cudaStream_t st)
 {
-    if (p->precision == 1) return launch_typed<double, 4>(p, p->dd, L, st);
-    if (p->NW == 5) return launch_typed<float, 5>(p, p->df, L, st);
-    if (p->NW == 6) return launch_typed<float, 6>(p, p->df, L, st);
-    if (p->NW == 8) return launch_typed<float, 8>(p, p->df, L, st);
-    return launch_typed<float, 4>(p, p->df, L, st);
+    if (p->precision == 1) return launch_typed<double, 4, 1>(p, p->dd, L, st);
+    if (p->NW == 5) return launch_typed<float, 5, 4>(p, p->df, L, st);
+    if (p->NW == 6) return launch_typed<float, 6, 3>(p, p->df, L, st);
+    if (p->NW == 8) return launch_typed<float, 8, 2>(p, p->df, L, st);
+    if (small_chain_ctas(p->geo, L.n_blocks)) return launch_typed<float, 4, 5>(p, p->df, L, st);
+    return launch_typed<float, 4, 4>(p, p->df, L, st);
 }
 
 }  // namespace pmf
