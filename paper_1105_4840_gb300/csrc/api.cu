@@ -434,6 +434,9 @@ static RunLaunch item_launch(const pmf_run *run, const RunItem &ri)
     L.abort = run->d_abort;
     L.wout = run->d_w;       // set for pulled runs only
     L.smd_vdt = run->smd_vdt;
+    for (int i = ri.w0; i < ri.w0 + ri.nw; ++i)
+        L.lambda_max = std::max({L.lambda_max, std::fabs(run->lambda[i]),
+                                 std::fabs(run->lambda[i] + run->smd_vdt * (double)run->nsteps[i])});
     // 1D runs: this item's block of the noise buffer
     L.noise = run->d_noise ? run->d_noise + (size_t)run->noise_steps * ri.w0 * run->replicas : nullptr;
     L.noise_steps = run->noise_steps;

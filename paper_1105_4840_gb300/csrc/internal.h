@@ -69,6 +69,7 @@ struct RunLaunch {
     // constant-velocity pulling (one window): the trap advances smd_vdt per
     // step after the equilibration; accumulated work recorded into wout
     double smd_vdt = 0;
+    double lambda_max = 0;  // 1D model: largest |trap centre| of the launch
     double *wout = nullptr;
     // 1D model: buffer for the per-step noise-and-trap terms q_n of noise_steps
     // steps of every simulation

@@ -7,16 +7,29 @@
 // Regrouped, x_{n+1} = x_n (cA x_n^2 + cB) + q_n with cA = -4a dt/gamma,
 // cB = 1 + (4a - k) dt/gamma and q_n = k lambda_n dt/gamma + amp xi_n.  q_n
 // does not depend on the trajectory, so a parallel pre-pass computes it for
-// a block of steps of every simulation; the sequential integration then costs
-// three FP64 operations per step, the rate at which this GPU's FP64 unit
-// retires them bounding a few hundred simulations.
+// a block of steps of every simulation; the integration is one dependent
+// chain per simulation, and its latency per step is the time of the run.
+//
+// Arithmetic of the chain.  This GPU's FP64 unit takes 64 cycles per operation
+// of a warp, dependent or not, so the three FP64 operations of a step cost 192
+// cycles.  Where the launch's parameters bound the motion, the chain runs in
+// 62-bit fixed point on the integer pipe instead (IMAD.WIDE: 5 cycles):
+// X = x 2^S with |x| < 2^b, S = 62 - b, and
+//   X' = X + Q + X w,  w = (cB - 1) + cA 4^b (X 2^-62)^2,
+// products of 62-bit numbers within a few units of 2^(b-62) (9e-19 for the
+// double well's b = 2), 1/128 of the FP64 rounding of a position near 1; the
+// results are no further from the exact map than FP64's.  A simulation that leaves |x| < 2^b redoes the
+// tile of steps it left in, and runs on, in FP64.
+#include <algorithm>
+#include <cmath>
+
 #include "common.cuh"
 #include "internal.h"
 
 namespace pmf {
 
 struct Od1dArgs {
-    double a, x0, k, kT, dt, gamma;
+    double x0, k;
     const double *lambda;
     const long long *nsteps_w, *nequil_w, *off_w, *tw;
     double *state;              // [n_rep][2]: x and the accumulated pulling work
@@ -31,7 +44,11 @@ struct Od1dArgs {
     long long window_steps;
     double *wout;               // constant-velocity pulling: work at the records
     double smd_vdt;             //   trap advance per step after the equilibration
-    const double *noise;        // [c1 - c0][n_rep] q_n of this launch's steps
+    long long *noise;           // [c1 - c0][n_rep] q_n of this launch's steps (fixed: q_n 2^S, else the double's bits)
+    int fixed, range_log2;      // fixed point: on, and b
+    double cA, cB1;             // -4a dt/gamma, (4a - k) dt/gamma
+    double amp, ck;             // sqrt(2 kT dt/gamma), k dt/gamma; fixed: times 2^S (set on the host: per thread
+                                // they took a sixth of the pre-pass's FP64 operations)
 };
 
 // Trap centre during step n of simulation rep: its window's lambda (the
@@ -48,7 +65,7 @@ __device__ __forceinline__ double trap_centre(const Od1dArgs &a, int rep, long l
 
 // q_n of every simulation for steps [c0, c1), one Philox block (four steps
 // of one simulation) per thread, stored [n - c0][rep].
-__global__ void od1d_noise_kernel(const Od1dArgs a, double *q)
+__global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
 {
     const long long nb = (a.c1 - a.c0 + 3) >> 2;  // c0 is a multiple of 4
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -59,94 +76,260 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, double *q)
     const Normal4<double> z =
         philox_normals<double>(a.seed, 0u, a.uid_base + (uint32_t)rep, (uint32_t)(n0 >> 2), kTagOStep);
     const double v[4] = {z.n0, z.n1, z.n2, z.n3};
-    const double dtg = a.dt / a.gamma, amp = sqrt(2.0 * a.kT * dtg), ck = a.k * dtg;
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
         const long long n = n0 + l;
-        if (n < a.c1) q[(n - a.c0) * a.n_rep + rep] = fma(amp, v[l], ck * trap_centre(a, rep, n));
+        if (n < a.c1) {
+            const double qn = fma(a.amp, v[l], a.ck * trap_centre(a, rep, n));
+            q[(n - a.c0) * a.n_rep + rep] = a.fixed ? __double2ll_rn(qn) : __double_as_longlong(qn);
+        }
     }
 }
 
-// One thread per simulation, steps [c0, c1): the parallel protocol (window
-// rep / R throughout), the sequential protocol (window = step / tau, Sec.
-// III (i)) or constant-velocity pulling (the trap at lambda_1 + vdt (n -
-// n_equil) from step n_equil on, the move before step n doing the work of
-// Eq. (9) at the current x).
-// First `done` count (steps completed in the window) > from at which a sample
-// is recorded: nequil + m stride, m >= 1.
-__device__ __forceinline__ long long next_sample(long long from, long long nequil, int stride)
+// A 62-bit fixed-point number as two 31-bit limbs, h 2^31 + l with
+// 0 <= l < 2^31.  a b 2^-62 of two such numbers (|a|, |b| < 2^62) is
+// a.h b.h + 2 (hi(a.h b.l) + hi(a.l b.h)), hi = the upper 32 bits of a 64-bit
+// product, within 5 units: the two cross products keep 30 bits each and the
+// product of the low limbs is dropped.
+struct Limbs {
+    int h, l;
+};
+__device__ __forceinline__ Limbs limbs(long long v) { return {(int)(v >> 31), (int)(v & 0x7fffffff)}; }
+__device__ __forceinline__ int mad_hi(int a, int b, int c)
 {
-    const long long m = from < nequil + stride ? 1 : (from - nequil) / stride + 1;
-    return nequil + m * stride;
+    int d;
+    asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c)  // wraps
+{
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ long long mul62_add(Limbs a, Limbs b, long long c)
+{
+    return mad_wide(mad_hi(a.l, b.h, __mulhi(a.h, b.l)), 2, mad_wide(a.h, b.h, c));
 }
 
-__global__ void od1d_kernel(const Od1dArgs a)
+struct FixedStep {
+    Limbs ca;      // cA 4^b 2^62
+    long long cb;  // (cB - 1) 2^62
+};
+// One step, X' = X + Q + X w, w = (cB - 1) + cA x^2: three products, 19
+// integer instructions with the sums folded into the multiply-adds (64-bit
+// products by limbs cost twice that, most of it shifts and splits).  Sums wrap
+// where a trajectory leaves the range; the caller discards that tile.
+__device__ __forceinline__ long long fixed_step(const FixedStep &f, long long X, long long q)
 {
-    const int rep = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rep >= a.n_rep) return;
+    const Limbs x = limbs(X);
+    const Limbs y = limbs(mad_wide(__mulhi(x.h, x.l), 4, (long long)x.h * x.h));
+    const Limbs w = limbs(mul62_add(f.ca, y, f.cb));
+    return mul62_add(w, x, (long long)((unsigned long long)X + (unsigned long long)q));
+}
+
+// 32 simulations per CTA, steps [c0, c1): the parallel protocol (window rep /
+// R throughout), the sequential protocol (window = step / tau, Sec. III (i))
+// or constant-velocity pulling (the trap at lambda_1 + vdt (n - n_equil) from
+// step n_equil on, the move before step n doing the work of Eq. (9) at the
+// current x).  Warp 0 integrates, lane = simulation, a tile of kTile steps at
+// a time from shared memory to shared memory; warps 1 - 3 meanwhile fetch the
+// next tile's q_n and turn the previous tile's positions into samples and
+// pulling work, so the dependent chain carries nothing else.  What bounds it is
+// that chain: 118 cycles a step by itself (a product of limbs is four dependent
+// 32 x 32 -> 64 multiplies of 9 - 12 cycles and a split), about 145 with the
+// tile's barrier; one thread per simulation in FP64 with loads and samples in
+// its loop took 403.  21 x 8 simulations x 2e4 steps, whole run with estimates:
+// 4.62 -> 1.80 ms; 256 pulled simulations x 4400 steps: 2.27 -> 0.75 ms.
+constexpr int kTile = 40;  // 41.5 KB of shared memory a CTA; 32 steps: 2.17 against 1.90 ms
+static_assert(kTile % 8 == 0, "unrolled by 8");
+constexpr int kOd1dThreads = 128;
+
+__global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
+{
+    __shared__ long long Q[2][kTile][32];      // q_n
+    __shared__ long long X[2][kTile + 1][32];  // positions before the tile's first step and after each
+    __shared__ unsigned dbl_mask[2];           // lanes whose tile is in FP64 (bits of doubles)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rep = blockIdx.x * 32 + lane;
+    const bool live = rep < a.n_rep;
     const int r = a.sequential ? rep : rep % a.replicas;
-    int w = a.sequential ? (int)(a.c0 / a.window_steps) : rep / a.replicas;
-    long long c1 = a.c1;
-    if (!a.sequential) c1 = c1 < a.nsteps_w[w] ? c1 : a.nsteps_w[w];
-    if (a.c0 >= c1) return;
-    double x = a.c0 == 0 ? (a.start ? a.start[rep] : a.x0) : a.state[2 * rep];
-    double W = a.c0 == 0 ? 0.0 : a.state[2 * rep + 1];
-    const double lam1 = a.lambda[0], dtg = a.dt / a.gamma;
-    const double cA = -4.0 * a.a * dtg, cB = 1.0 + (4.0 * a.a - a.k) * dtg;
-    // per-window quantities, refreshed when a sequential run enters a window
-    long long origin = a.sequential ? (long long)w * a.window_steps : 0;
-    long long win_end = a.sequential ? origin + a.window_steps : c1;
-    long long nequil = a.nequil_w[w];
-    double lam = a.lambda[w];
-    long long base = a.off_w[w] + (long long)r * a.tw[w];
-    long long next = next_sample(a.c0 - origin, nequil, a.stride);  // in the window's step count
-    if (a.wout && a.c0 - 1 > nequil) lam = lam1 + a.smd_vdt * (double)(a.c0 - 1 - nequil);  // pulled so far
-    // q_n in blocks of kPre steps, the next block's loads issued before the
-    // current block is integrated (the dependent steps are short; an L2 load
-    // per step would otherwise stall every step)
-    constexpr int kPre = 8;
-    const double *xi = a.noise + rep;
-    double cur[kPre], nxt[kPre];
-#pragma unroll
-    for (int j = 0; j < kPre; ++j) cur[j] = a.c0 + j < c1 ? xi[(long long)j * a.n_rep] : 0.0;
-    for (long long n0 = a.c0; n0 < c1; n0 += kPre) {
-#pragma unroll
-        for (int j = 0; j < kPre; ++j) {
-            const long long m = n0 + kPre + j;
-            nxt[j] = m < c1 ? xi[(m - a.c0) * a.n_rep] : 0.0;
+    const int w = a.sequential || !live ? 0 : rep / a.replicas;
+    // this simulation's last step (its window's step count)
+    long long end = a.c1;
+    if (!a.sequential && live) end = end < a.nsteps_w[w] ? end : a.nsteps_w[w];
+    if (!live || end < a.c0) end = a.c0;
+    const double scale = scalbn(1.0, 62 - a.range_log2), unit = scalbn(1.0, a.range_log2 - 62);
+    const double cA = a.cA, cB1 = a.cB1, cB = 1.0 + cB1;
+    const long long tiles = (a.c1 - a.c0 + kTile - 1) / kTile;
+
+    auto load_tile = [&](long long i, int row, int step) {
+        const long long n0 = i * kTile;
+        for (int s = row; s < kTile; s += step)
+            if (live && n0 + s < a.c1 - a.c0) Q[i & 1][s][lane] = a.noise[(n0 + s) * a.n_rep + rep];
+    };
+
+    // warp 0: the position, in fixed point or (dbl) FP64
+    FixedStep f{};
+    long long Xi = 0;
+    double x = 0.0;
+    bool dbl = true;
+    if (warp == 0 && live) {
+        x = a.c0 == 0 ? (a.start ? a.start[rep] : a.x0) : a.state[2 * rep];
+        if (a.fixed) {
+            f.ca = limbs(__double2ll_rn(scalbn(cA, 62 + 2 * a.range_log2)));
+            f.cb = __double2ll_rn(scalbn(cB1, 62));
+            if (fabs(x) < scalbn(1.0, a.range_log2)) {
+                Xi = __double2ll_rn(x * scale);
+                dbl = false;
+            }
         }
-#pragma unroll
-        for (int j = 0; j < kPre; ++j) {
-        const long long n = n0 + j;
-        if (n >= c1) break;
-        if (n == win_end) {  // sequential protocol: the trap moves to the next window
-            ++w;
-            origin = n;
-            win_end = n + a.window_steps;
-            nequil = a.nequil_w[w];
-            lam = a.lambda[w];
-            base = a.off_w[w] + (long long)r * a.tw[w];
-            next = next_sample(0, nequil, a.stride);
-        }
-        if (a.wout && n > nequil) {
-            const double lo = lam;
-            lam = lam1 + a.smd_vdt * (double)(n - nequil);
-            W += 0.5 * a.k * (lam - lo) * (lam + lo - 2.0 * x);
-        }
-        x = fma(x, fma(cA, x * x, cB), cur[j]);
-        if (n + 1 - origin == next) {
-            const long long at = base + (next - nequil) / a.stride - 1;
-            a.xout[at] = (float)x;
-            if (a.wout) a.wout[at] = W;
-            next += a.stride;
-        }
-        }
-#pragma unroll
-        for (int j = 0; j < kPre; ++j) cur[j] = nxt[j];
     }
-    if (!isfinite(x)) atomicOr(a.err, kErrNonFinite);
-    a.state[2 * rep] = x;
-    a.state[2 * rep + 1] = W;
+    auto integrate = [&](long long i) {
+        const long long n0 = a.c0 + i * kTile;
+        const int b = (int)(i & 1);
+        const int lim = end <= n0 ? 0 : (end - n0 < kTile ? (int)(end - n0) : kTile);
+        const long long X0 = Xi;
+        bool redo = dbl && lim > 0;
+        if (!dbl) {
+            X[b][0][lane] = Xi;
+            int guard = 0;  // sign bit: a position outside [-2^62, 2^62)
+            if (__all_sync(__activemask(), lim == kTile)) {
+#pragma unroll 8
+                for (int s = 0; s < kTile; ++s) {
+                    Xi = fixed_step(f, Xi, Q[b][s][lane]);
+                    X[b][s + 1][lane] = Xi;
+                    guard |= (int)(Xi >> 32) + 0x40000000;
+                }
+            } else {
+                for (int s = 0; s < lim; ++s) {
+                    Xi = fixed_step(f, Xi, Q[b][s][lane]);
+                    X[b][s + 1][lane] = Xi;
+                    guard |= (int)(Xi >> 32) + 0x40000000;
+                }
+            }
+            if (guard < 0) {
+                x = (double)X0 * unit;
+                dbl = redo = true;
+            }
+        }
+        if (redo) {
+            X[b][0][lane] = __double_as_longlong(x);
+#pragma unroll 4
+            for (int s = 0; s < lim; ++s) {
+                const long long qb = Q[b][s][lane];
+                x = fma(x, fma(cA, x * x, cB), a.fixed ? (double)qb * unit : __longlong_as_double(qb));
+                X[b][s + 1][lane] = __double_as_longlong(x);
+            }
+        }
+        __syncwarp();
+        const unsigned mask = __ballot_sync(0xffffffffu, dbl);
+        if (lane == 0) dbl_mask[b] = mask;
+    };
+
+    // warps 1 - 3: the records of a finished tile, record number `at` of a
+    // window by helper at mod 3; no division in the loop.  rec: step whose end
+    // the helper's next record is taken at.
+    const int helper = warp - 1;
+    constexpr int kHelpers = kOd1dThreads / 32 - 1;
+    int ww = w;
+    long long rec = 0, at = 0, base = 0, wend = 0;
+    auto enter_window = [&](int window, long long from) {
+        ww = window;
+        const long long origin = a.sequential ? (long long)ww * a.window_steps : 0;
+        const long long past = from - origin - a.nequil_w[ww];
+        const long long at0 = past > 0 ? past / a.stride : 0;  // records taken before step `from`
+        at = at0 + (helper + kHelpers - at0 % kHelpers) % kHelpers;
+        rec = origin + a.nequil_w[ww] + (at + 1) * a.stride - 1;
+        base = a.off_w[ww] + (long long)r * a.tw[ww];
+        wend = a.sequential ? origin + a.window_steps : end;
+    };
+    // pulling work: W after the trap's first moves0 moves, and since then the
+    // sum of X - lambda_1 in two 32-bit halves (every helper keeps it, each
+    // converts for its own records)
+    double W = 0.0;
+    long long acc_h = 0, moves0 = 0, moves = 0;
+    unsigned long long acc_l = 0;
+    const double lam1 = a.lambda[0], kv = a.k * a.smd_vdt;
+    const long long L1 = a.fixed ? __double2ll_rn(lam1 * scale) : 0;
+    if (warp > 0 && live) {
+        enter_window(a.sequential ? (int)(a.c0 / a.window_steps) : w, a.c0);
+        if (a.wout) {
+            W = a.c0 == 0 ? 0.0 : a.state[2 * rep + 1];
+            moves = a.c0 - 1 - a.nequil_w[0];
+            moves0 = moves = moves > 0 ? moves : 0;
+        }
+    }
+    // sum over the moves m of k vdt (lambda_1 + vdt (m - 1/2) - x)
+    auto fixed_work = [&] {
+        const double m = (double)moves, m0 = (double)moves0;
+        const double sum = ((double)acc_h * 4294967296.0 + (double)acc_l) * unit;
+        return W + kv * (0.5 * a.smd_vdt * (m * m - m0 * m0) - sum);
+    };
+    auto records = [&](long long i) {
+        if (!live) return;  // (such a lane has no window to record in)
+        const int b = (int)(i & 1);
+        const bool d = (dbl_mask[b] >> lane) & 1;
+        const long long n0 = a.c0 + i * kTile, stop = end < n0 + kTile ? end : n0 + kTile;
+        long long n = n0;  // positions before this step are in the work
+        if (a.wout && d && moves != moves0) {  // FP64 from here on
+            W = fixed_work();
+            moves0 = moves;
+            acc_h = 0;
+            acc_l = 0;
+        }
+        const long long move1 = a.wout ? a.nequil_w[0] + 1 : 0;  // the step before which the trap first moves
+        auto moves_to = [&](long long to) {                      // the trap's moves before steps [n, to)
+            if (n < move1) n = move1;
+            for (; n < to; ++n) {
+                const long long v = X[b][n - n0][lane];
+                moves = n - move1 + 1;
+                if (d) {
+                    const double lo = lam1 + a.smd_vdt * (double)(moves - 1), hi = lam1 + a.smd_vdt * (double)moves;
+                    W += 0.5 * a.k * (hi - lo) * (hi + lo - 2.0 * __longlong_as_double(v));
+                    moves0 = moves;
+                } else {
+                    const long long e = v - L1;
+                    acc_h += e >> 32;
+                    acc_l += (unsigned)e;
+                }
+            }
+        };
+        for (;;) {
+            for (const long long seg = wend < stop ? wend : stop; rec < seg; rec += kHelpers * a.stride, at += kHelpers) {
+                const long long v = X[b][rec - n0 + 1][lane];
+                a.xout[base + at] = d ? (float)__longlong_as_double(v) : (float)v * (float)unit;
+                if (a.wout) {
+                    moves_to(rec + 1);
+                    a.wout[base + at] = d ? W : fixed_work();
+                }
+            }
+            if (!a.sequential || wend >= stop) break;
+            enter_window(ww + 1, wend);
+        }
+        if (a.wout) moves_to(stop);
+    };
+
+    load_tile(0, warp, kOd1dThreads / 32);
+    __syncthreads();
+    for (long long i = 0; i <= tiles; ++i) {
+        if (warp == 0) {
+            if (i < tiles) integrate(i);
+        } else {
+            if (i + 1 < tiles) load_tile(i + 1, warp - 1, kOd1dThreads / 32 - 1);
+            if (i > 0) records(i - 1);
+        }
+        __syncthreads();
+    }
+    if (!live || end <= a.c0) return;
+    if (warp == 0) {
+        if (!dbl) x = (double)Xi * unit;
+        if (!isfinite(x)) atomicOr(a.err, kErrNonFinite);
+        a.state[2 * rep] = x;
+        if (!a.wout) a.state[2 * rep + 1] = 0.0;
+    } else if (warp == 1 && a.wout) {
+        a.state[2 * rep + 1] = moves != moves0 ? fixed_work() : W;
+    }
 }
 
 long long od1d_noise_steps(int n_rep)
@@ -163,12 +346,8 @@ cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cuda
         return cudaErrorInvalidValue;
     if (L.sequential && L.window_steps < 1) return cudaErrorInvalidValue;
     Od1dArgs a{};
-    a.a = m.a;
     a.x0 = m.x0;
     a.k = L.k;
-    a.kT = L.kT;
-    a.dt = L.dt;
-    a.gamma = L.gamma;
     a.lambda = L.lambda;
     a.nsteps_w = L.nsteps_w;
     a.nequil_w = L.nequil_w;
@@ -187,23 +366,37 @@ cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cuda
     a.window_steps = L.window_steps;
     a.wout = L.wout;
     a.smd_vdt = L.smd_vdt;
-    a.noise = L.noise;
-    // few simulations: spread them over the SMs (one warp each) rather than
-    // packing them into a few CTAs; many: 128 threads per CTA
-    int dev = 0, sms = 1;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return cudaGetLastError();
-    const int per_sm = (n_rep + sms - 1) / sms;
-    const int threads = per_sm <= 32 ? 32 : (per_sm <= 64 ? 64 : 128);
+    a.noise = reinterpret_cast<long long *>(L.noise);
+    // Fixed point where |x| < 2^b holds the traps, the start, the wells and six
+    // widths of the trap, and where one step from inside cannot wrap a 64-bit
+    // sum (which also bounds every coefficient): FP64 otherwise, for instance
+    // for time steps near the scheme's stability limit.  Box-Muller's normals
+    // stay below sqrt(66 ln 2) < 6.8.
+    const double dtg = L.dt / L.gamma, reach = std::max({L.lambda_max, std::fabs(m.x0), m.a != 0.0 ? 1.0 : 0.0}) + 6.0 * std::sqrt(L.kT / L.k);
+    const double cA = std::fabs(4.0 * m.a * dtg), cB1 = std::fabs((4.0 * m.a - L.k) * dtg);
+    const double qmax = 6.8 * std::sqrt(2.0 * L.kT * dtg) + L.k * dtg * L.lambda_max;
+    if (std::isfinite(reach) && reach > 0 && std::isfinite(cA) && std::isfinite(cB1) && std::isfinite(qmax)) {
+        int b = 0;
+        std::frexp(reach, &b);  // reach <= 2^b
+        if (b >= -30 && b <= 30 && cB1 + std::ldexp(cA, 2 * b) + std::ldexp(qmax, -b) < 0.99) {
+            a.fixed = 1;
+            a.range_log2 = b;
+        }
+    }
+    a.cA = -4.0 * m.a * dtg;
+    a.cB1 = (4.0 * m.a - L.k) * dtg;
+    const double scale = a.fixed ? std::ldexp(1.0, 62 - a.range_log2) : 1.0;
+    a.amp = std::sqrt(2.0 * L.kT * dtg) * scale;
+    a.ck = L.k * dtg * scale;
     for (long long c0 = L.step_begin; c0 < L.step_end; c0 += L.noise_steps) {
         const long long c1 = c0 + L.noise_steps < L.step_end ? c0 + L.noise_steps : L.step_end;
         const long long cells = ((c1 - c0 + 3) >> 2) * n_rep;
         a.c0 = c0;
         a.c1 = c1;
-        od1d_noise_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(a, L.noise);
+        od1d_noise_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, st>>>(a, a.noise);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        od1d_kernel<<<(n_rep + threads - 1) / threads, threads, 0, st>>>(a);
+        od1d_kernel<<<(n_rep + 31) / 32, kOd1dThreads, 0, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
