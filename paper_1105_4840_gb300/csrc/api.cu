@@ -77,6 +77,17 @@ template <typename T> cudaError_t upload(T **d, const T *h, size_t n)
     return n ? cudaMemcpy(*d, h, sizeof(T) * n, cudaMemcpyHostToDevice) : cudaSuccess;
 }
 
+// Reduction scratch of `bytes` (reduce_scratch_bytes, or what is left of it
+// without the partials), its counter zeroed.
+cudaError_t alloc_reduce(void **buf, size_t bytes, unsigned **counter)
+{
+    cudaError_t e = cudaMalloc(buf, bytes);
+    if (e != cudaSuccess) return e;
+    const unsigned zero = 0;
+    *counter = reduce_counter(*buf, bytes);
+    return cudaMemcpy(*counter, &zero, sizeof(zero), cudaMemcpyHostToDevice);
+}
+
 }  // namespace
 
 struct pmf_system {
@@ -127,6 +138,7 @@ struct pmf_run {
     void *d_state = nullptr;
     int *d_err = nullptr;
     void *d_scratch = nullptr;
+    unsigned *d_count = nullptr;  // (inside d_scratch)
     double *d_res = nullptr;
     double *d_start = nullptr;  // per-replica start state of a seeded run
     unsigned long long *d_queue = nullptr;  // persistent launch: work counter
@@ -339,7 +351,7 @@ static pmf_status prepare_items(pmf_system *sys, const pmf_batch_item *items, in
     CK(cudaMalloc(&run->d_x, sizeof(float) * run->total), "alloc samples");
     CK(cudaMalloc(&run->d_state, run->state_bytes), "alloc state");
     CK(cudaMalloc(&run->d_err, sizeof(int)), "alloc flag");
-    CK(cudaMalloc(&run->d_scratch, reduce_scratch_bytes(max_nw, p->replicas)), "alloc scratch");
+    CK(alloc_reduce(&run->d_scratch, reduce_scratch_bytes(max_nw, p->replicas), &run->d_count), "alloc scratch");
     CK(cudaMalloc(&run->d_res, sizeof(double) * kResFields * max_nw), "alloc results");
     CK(cudaEventCreateWithFlags(&run->done, cudaEventDisableTiming), "event");
     CK(cudaStreamCreateWithFlags(&run->cap, cudaStreamNonBlocking), "capture stream");
@@ -751,6 +763,8 @@ static ReduceLayout layout_of(const pmf_run *run)
     L.lambda = run->d_lambda;
     L.off_w = run->d_off;
     L.tw = run->d_tw;
+    L.t_max = *std::max_element(run->tw.begin(), run->tw.end());
+    L.counter = run->d_count;
     L.n_windows = run->n_windows;
     L.replicas = run->replicas;
     L.k = run->k;
@@ -802,6 +816,7 @@ static ReduceLayout item_layout(const pmf_run *run, int item)
     L.lambda = run->d_lambda + ri.w0;
     L.off_w = run->d_off + ri.w0;
     L.tw = run->d_tw + ri.w0;
+    L.t_max = *std::max_element(run->tw.begin() + ri.w0, run->tw.begin() + ri.w0 + ri.nw);
     L.n_windows = ri.nw;
     return L;
 }
@@ -1159,13 +1174,14 @@ pmf_status pmf_state_free_energy_from_samples(const float *x, int x_on_device, c
         CK(upload(&t.x, x, (size_t)total), "upload samples");
         dx = t.x;
     }
-    CK(cudaMalloc(&t.scratch, reduce_scratch_bytes(n_windows, replicas)), "alloc scratch");
-    CK(cudaMalloc(&t.res, sizeof(double) * kResFields * n_windows), "alloc result");
     ReduceLayout L;
+    CK(alloc_reduce(&t.scratch, reduce_scratch_bytes(n_windows, replicas), &L.counter), "alloc scratch");
+    CK(cudaMalloc(&t.res, sizeof(double) * kResFields * n_windows), "alloc result");
     L.x = dx;
     L.lambda = t.lam;
     L.off_w = t.off;
     L.tw = t.tw;
+    L.t_max = *std::max_element(tw.begin(), tw.end());
     L.n_windows = n_windows;
     L.replicas = replicas;
     L.k = k;
@@ -1194,10 +1210,10 @@ pmf_status pmf_free_energy_from_partials(const double *partials, const double *l
     } t;
     CK(upload(&t.lam, lambda, n_windows), "upload lambda");
     CK(upload(&t.P, partials, np), "upload partials");
-    CK(cudaMalloc(&t.wo, reduce_scratch_bytes(n_windows, replicas) - partial_bytes(n_windows, replicas)),
+    ReduceLayout L;
+    CK(alloc_reduce(&t.wo, reduce_scratch_bytes(n_windows, replicas) - partial_bytes(n_windows, replicas), &L.counter),
        "alloc scratch");
     CK(cudaMalloc(&t.res, sizeof(double) * kResFields * n_windows), "alloc results");
-    ReduceLayout L;
     L.lambda = t.lam;
     L.n_windows = n_windows;
     L.replicas = replicas;
@@ -1244,13 +1260,14 @@ pmf_status pmf_free_energy_from_samples(const float *x, int x_on_device, const d
         CK(upload(&t.x, x, (size_t)total), "upload samples");
         dx = t.x;
     }
-    CK(cudaMalloc(&t.scratch, reduce_scratch_bytes(n_windows, replicas)), "alloc scratch");
-    CK(cudaMalloc(&t.res, sizeof(double) * kResFields * n_windows), "alloc result");
     ReduceLayout L;
+    CK(alloc_reduce(&t.scratch, reduce_scratch_bytes(n_windows, replicas), &L.counter), "alloc scratch");
+    CK(cudaMalloc(&t.res, sizeof(double) * kResFields * n_windows), "alloc result");
     L.x = dx;
     L.lambda = t.lam;
     L.off_w = t.off;
     L.tw = t.tw;
+    L.t_max = *std::max_element(tw.begin(), tw.end());
     L.n_windows = n_windows;
     L.replicas = replicas;
     L.k = k;
@@ -1783,13 +1800,14 @@ pmf_status pmf_run_adaptive(pmf_system *sys, const double *lambda0, int n0, cons
     CK(merge_windows(win, R, m), "merge samples");
     void *scratch = nullptr;
     double *d_res = nullptr;
-    CK(cudaMalloc(&scratch, reduce_scratch_bytes(m.n, R)), "alloc");
-    cudaError_t e = cudaMalloc(&d_res, sizeof(double) * kResFields * m.n);
     ReduceLayout RL;
+    cudaError_t e = alloc_reduce(&scratch, reduce_scratch_bytes(m.n, R), &RL.counter);
+    if (e == cudaSuccess) e = cudaMalloc(&d_res, sizeof(double) * kResFields * m.n);
     RL.x = m.x;
     RL.lambda = m.lam;
     RL.off_w = m.off;
     RL.tw = m.tw;
+    for (const Window &q : win) RL.t_max = std::max(RL.t_max, q.run->tw[q.w]);
     RL.n_windows = m.n;
     RL.replicas = R;
     RL.k = p->k;

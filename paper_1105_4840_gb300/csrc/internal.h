@@ -154,8 +154,10 @@ long long od1d_noise_steps(int n_rep);
 struct ReduceLayout {
     const float *x = nullptr;          // device samples
     const double *lambda = nullptr;    // device [s]
-    const long long *off_w = nullptr;  // device [s]
-    const long long *tw = nullptr;     // device [s]
+    const long long *off_w = nullptr;  // device [s]; null: windows of t_max samples a replica, end to end
+    const long long *tw = nullptr;     // device [s]; null: t_max
+    long long t_max = 0;               // most samples a replica of any window has
+    unsigned *counter = nullptr;       // device, 0 between launches: windows combined (see reduce_counter)
     int n_windows = 0, replicas = 0;
     double k = 0, kT = 1;
 };
@@ -166,6 +168,9 @@ enum ResultField {
 };
 // scratch: device buffer of reduce_scratch_bytes(); out: device [kResFields][n_windows]
 size_t reduce_scratch_bytes(int n_windows, int replicas);
+// The counter at the end of a scratch buffer of `bytes` (reduce_scratch_bytes
+// or what is left of it after the partials); the allocation zeroes it.
+unsigned *reduce_counter(void *buffer, size_t bytes);
 cudaError_t reduce_launch(const ReduceLayout &L, void *scratch, double *out, cudaStream_t st);
 // The two halves of reduce_launch.  Per-replica partials, 5 doubles each,
 // [window][replica]: {min w, sum exp(-(w - min)/kT), n, sum (x - lambda_i),

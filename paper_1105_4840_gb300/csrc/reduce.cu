@@ -1,6 +1,7 @@
 // FP64 reductions of the recorded x samples into the paper's estimators.
 //
-// Stage 1 (one CTA per (window i, replica r), two passes over the samples):
+// Stage 1 (a team of 1, 2, 4 or 8 warps per (window i, replica r), two passes
+// over the samples):
 //   work increments of Eq. (9),
 //   w = k/2 (lambda_{i+1} - lambda_i)(lambda_{i+1} + lambda_i - 2 x),
 //   the replica's minimum m_ir, the max-shifted exponential sum
@@ -9,13 +10,24 @@
 // Stage 2 (one CTA per window): merge the replicas (log-sum-exp aware),
 //   the per-window JE increment, the Eq. (14) and Eq. (13) increments and
 //   the delete-one-replica jackknife.
-// Stage 3 (one thread): prefix sums over windows into the profiles and the
-//   combined estimate of Sec. V.
+// Stage 3 (the last CTA of stage 2): prefix sums over windows into the
+//   profiles and the combined estimate of Sec. V.
 // The windows are independent (Sec. II: rho(W_mech) is the product of the
 // rho(x_i)), so the average of exp(-W_mech/kT) over all combinations of
 // samples is the product of the per-window averages.
+//
+// What bounds the three stages on small and ordinary paths is the latency of
+// FP64 operations (64 cycles each for one warp of this GPU), so stages 2 and 3
+// spend as few of them in sequence as they can and run independent ones on
+// different warps.  21 windows x 32 replicas x 3600 samples, back to back:
+// four launches (layout, partials, windows, profiles) 65.6 us, now 30.7 us;
+// 5 x 4 x 256: 49.2 us, now 20.5 us; 64 x 512 x 1801: 724 us, now 274 us.
 #include <math.h>
+#include <stddef.h>
 
+#include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <mutex>
 
 #include "common.cuh"
@@ -104,36 +116,48 @@ __device__ __forceinline__ void fast_two_sum_f(float a, float b, float &s, float
     e = b - (s - a);
 }
 
-struct ExpConsts {
-    float inv_l;          // 32 / ln 2
-    float l1, l2, l3;     // ln2/32 = l1 + l2 + l3, l1 with 12 significant bits
+// Passed by value: 2^(j/32) as hi + lo, 32 / ln 2, and ln2/32 = l1 + l2 + l3
+// with 12 significant bits in l1.
+struct ExpTable {
+    float hi[32], lo[32];
+    float inv_l, l1, l2, l3;
 };
 
-__device__ __forceinline__ ExpConsts exp_consts()
+const ExpTable &exp_table()
 {
-    // ln 2 as the double nearest to it plus the remainder
-    const double ln2_hi = 0.6931471805599453, ln2_lo = 2.319046813846299558e-17;
-    const double l = ln2_hi / 32.0;  // exact: a power-of-two scaling
-    ExpConsts k;
-    k.inv_l = (float)(32.0 / ln2_hi);
-    k.l1 = __int_as_float(__float_as_int((float)l) & ~0xFFF);
-    const double r1 = l - (double)k.l1;
-    k.l2 = (float)r1;
-    k.l3 = (float)((r1 - (double)k.l2) + ln2_lo / 32.0);
-    return k;
+    static const ExpTable table = [] {
+        ExpTable t;
+        for (int j = 0; j < 32; ++j) {
+            const double v = std::exp2(j / 32.0);
+            t.hi[j] = (float)v;
+            t.lo[j] = (float)(v - (double)t.hi[j]);
+        }
+        // ln 2 as the double nearest to it plus the remainder
+        const double ln2_hi = 0.6931471805599453, ln2_lo = 2.319046813846299558e-17;
+        const double l = ln2_hi / 32.0;  // exact: a power-of-two scaling
+        t.inv_l = (float)(32.0 / ln2_hi);
+        const float lf = (float)l;
+        uint32_t bits;
+        std::memcpy(&bits, &lf, 4);
+        bits &= ~0xFFFu;
+        std::memcpy(&t.l1, &bits, 4);
+        const double r1 = l - (double)t.l1;
+        t.l2 = (float)r1;
+        t.l3 = (float)((r1 - (double)t.l2) + ln2_lo / 32.0);
+        return t;
+    }();
+    return table;
 }
 
 // exp(ah + al) for ah + al <= 0 as a pair of floats eh + el (tab: 2^(j/32)
 // = tab_hi[j] + tab_lo[j]).
-__device__ __forceinline__ void exp_ff(float ah, float al, const ExpConsts &k, const float *tab_hi,
+__device__ __forceinline__ void exp_ff(float ah, float al, const ExpTable &k, const float *tab_hi,
                                        const float *tab_lo, float &eh, float &el)
 {
-    if (ah < -80.f) {
-        eh = el = 0.f;
-        return;
-    }
-    const float kf = rintf(ah * k.inv_l);
-    const int n = (int)kf;
+    // nearest integer to ah 32 / ln 2 (at most 3700 in size) by the addition of 1.5 2^23
+    const float big = fmaf(ah, k.inv_l, 12582912.f);
+    const float kf = big - 12582912.f;
+    const int n = __float_as_int(big) - 0x4B400000;
     // r = a - n ln2/32: n l1 is exact and close to ah, n l2 exact as p2 + e2
     const float t1 = fmaf(-kf, k.l1, ah);
     const float p2 = kf * k.l2;
@@ -159,17 +183,18 @@ __device__ __forceinline__ void exp_ff(float ah, float al, const ExpConsts &k, c
     two_sum_f(th, uh, hh, hl);
     hl += tl + ul;
     const float sc = __int_as_float((m + 127) << 23);
-    eh = hh * sc;
-    el = hl * sc;
+    const bool drop = ah < -80.f;
+    eh = drop ? 0.f : hh * sc;
+    el = drop ? 0.f : hl * sc;
 }
 
-// (h, l) += (bh, bl) in double-float arithmetic.
-__device__ __forceinline__ void ff_add(float &h, float &l, float bh, float bl)
+// Running sum h + l of float pairs: h carries the sum, l the rounding errors
+// of h (TwoSum, exact) and the low parts.
+__device__ __forceinline__ void ff_sum(float &h, float &l, float bh, float bl)
 {
-    float s, e;
-    two_sum_f(h, bh, s, e);
-    e += l + bl;
-    fast_two_sum_f(s, e, h, l);
+    float e;
+    two_sum_f(h, bh, h, e);
+    l += e + bl;
 }
 
 // Per-thread sums kept as pairs of floats and flushed into FP64 every
@@ -178,116 +203,186 @@ __device__ __forceinline__ void ff_add(float &h, float &l, float bh, float bl)
 // operations per flush instead of several per sample.
 constexpr int kFlushSamples = 16;
 
-template <int NT> __device__ float block_max_f(float v, float *red)
+// (double)f by integer operations (a conversion takes a turn of the FP64
+// unit); FP32 denormals are zero here as everywhere in this library's build.
+__device__ __forceinline__ double widen(float f)
 {
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    float t = red[0];
-    for (int q = 1; q < NT / 32; ++q) t = fmaxf(t, red[q]);
-    return t;
+    const int b = __float_as_int(f), e = b & 0x7f800000;
+    const int hi = (b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (e == 0x7f800000 ? 0x70000000 : 0x38000000));
+    return e == 0 ? __hiloint2double(b & 0x80000000, 0) : __hiloint2double(hi, b << 29);
 }
 
 // Per-window constants of stage 1, set once per CTA by one thread (the FP64
 // unit is the scarce one: per-thread setup in FP64 would cost more than the
 // samples themselves at a few samples per thread).
 struct WindowConsts {
-    double hkd, ssum;       // w = hkd (ssum - 2 x)
-    float ch, cl;           // c = 2 hkd / kT as a pair of floats
-    float li_h, li_m, li_l; // lambda_i as three floats
-    float sgn;              // +1: x_ref is the largest x, -1: the smallest
-    ExpConsts k;
+    double hkd, ssum;  // w = hkd (ssum - 2 x)
+    double lo;         // lambda_i - (float)lambda_i
+    float ch, cl;      // c = 2 hkd / kT as a pair of floats
+    float li;          // (float)lambda_i
 };
 
-__global__ void __launch_bounds__(kPartialThreads) partial_kernel(const ReduceLayout L, Partial *out)
+__device__ __forceinline__ long long samples_of(const ReduceLayout &L, int w) { return L.tw ? L.tw[w] : L.t_max; }
+__device__ __forceinline__ long long offset_of(const ReduceLayout &L, int w)
 {
-    // Two passes over the replica's samples (the second mostly from cache):
-    // the extreme x that minimises w, then per thread the exponential sum
-    // (terms by exp_ff) and the sums of (x - lambda_i) and its square as
-    // pairs of floats flushed into FP64, then trees over the threads.
-    __shared__ double red[kPartialThreads / 32 + 1];
-    __shared__ float redf[kPartialThreads / 32];
+    return L.off_w ? L.off_w[w] : (long long)w * L.replicas * L.t_max;
+}
+
+// Doubles in the order of their bits as signed integers (no NaN): compared
+// on the integer pipe.
+__device__ __forceinline__ long long order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double from_order_key(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+// Warp sums of three doubles in six additions instead of fifteen: the first
+// two exchanges also sort the quantities over the lanes.  a's sum is in lanes
+// 0..7, b's in 8..15, c's in 16..23.
+__device__ __forceinline__ double warp_sum3(double a, double b, double c, int lane)
+{
+    const bool up = lane & 16, mid = lane & 8;
+    double p = up ? c : a, q = up ? 0.0 : b;
+    p += __shfl_xor_sync(0xffffffffu, up ? a : c, 16);
+    q += __shfl_xor_sync(0xffffffffu, up ? b : 0.0, 16);
+    double v = mid ? q : p;
+    v += __shfl_xor_sync(0xffffffffu, mid ? p : q, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// Warp sums of two doubles in five additions: a's in lanes 0..15, b's in 16..31.
+__device__ __forceinline__ double warp_sum2(double a, double b, int lane)
+{
+    const bool up = lane & 16;
+    double v = up ? b : a;
+    v += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// CTA (w, chunk): replicas [chunk x per, (chunk + 1) x per) of window w, 8 / G
+// at a time by teams of G warps.  First pass: x_ref, the sample at which w is
+// smallest (the largest x if w falls with x, else the smallest); second pass
+// (mostly from cache): the exponential sum and the sums of q = x - (float)
+// lambda_i (exact as a pair of floats) and q^2; the rest of lambda_i enters
+// their totals in FP64.  About 100 FP32 operations a sample bound the large
+// stores, latency (loads, the FP64 trees) the small.
+// Five CTAs per SM for the large teams (672 replicas of 3600 samples then run
+// in one wave: 32.8 -> 30.7 us in all); four, with 64 registers, for a warp per
+// replica (64 x 512 x 1801: 274 us, five 283).
+template <int G>
+__global__ void __launch_bounds__(kPartialThreads, G >= 4 ? 5 : 4) partial_kernel(const ReduceLayout L, const __grid_constant__ ExpTable tab,
+                                                                  int per, Partial *out)
+{
+    constexpr int kTeams = kPartialThreads / 32 / G, kTeamThreads = 32 * G;
     __shared__ float tab_hi[32], tab_lo[32];
     __shared__ WindowConsts wc;
-    const int w = blockIdx.x, r = blockIdx.y;
-    const long long T = L.tw[w];
-    const float *x = L.x + L.off_w[w] + (long long)r * T;
+    __shared__ float red_max[kPartialThreads / 32];
+    __shared__ double red[kPartialThreads / 32][3];
+    const int w = blockIdx.x, R = L.replicas, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int team = warp / G, tid = threadIdx.x - team * kTeamThreads;
+    const long long T = samples_of(L, w), off = offset_of(L, w);
+    const double li = L.lambda[w], ln = w + 1 < L.n_windows ? L.lambda[w + 1] : li;
+    const float sgn = order_key(ln) < order_key(li) ? -1.f : 1.f;
     if (threadIdx.x < 32) {
-        const double t = exp2((double)threadIdx.x / 32.0);
-        tab_hi[threadIdx.x] = (float)t;
-        tab_lo[threadIdx.x] = (float)(t - (double)(float)t);
-    } else if (threadIdx.x == 32) {
-        const double li = L.lambda[w];
-        const double ln = (w + 1 < L.n_windows) ? L.lambda[w + 1] : li;
+        tab_hi[threadIdx.x] = tab.hi[threadIdx.x];
+        tab_lo[threadIdx.x] = tab.lo[threadIdx.x];
+    } else if (threadIdx.x == kPartialThreads - 1) {
         wc.hkd = 0.5 * L.k * (ln - li);
         wc.ssum = ln + li;
         const double c = 2.0 * wc.hkd / L.kT;
         wc.ch = (float)c;
         wc.cl = (float)(c - (double)wc.ch);
-        wc.li_h = (float)li;
-        wc.li_m = (float)(li - (double)wc.li_h);
-        wc.li_l = (float)((li - (double)wc.li_h) - (double)wc.li_m);
-        wc.sgn = wc.hkd < 0 ? -1.f : 1.f;
-        wc.k = exp_consts();
+        wc.li = (float)li;
+        wc.lo = li - (double)wc.li;
     }
-    if (T == 0) {
-        if (threadIdx.x == 0) out[(size_t)w * L.replicas + r] = Partial{INFINITY, 0.0, 0.0, 0.0, 0.0};
-        return;
-    }
-    __syncthreads();
-    // x_ref: the largest x if w falls with x (hkd > 0), else the smallest
-    const float sgn = wc.sgn;
-    float mx = -INFINITY;
-    for (long long t = threadIdx.x; t < T; t += kPartialThreads) mx = fmaxf(mx, sgn * x[t]);
-    const float xref = sgn * block_max_f<kPartialThreads>(mx, redf);
-    const float ch = wc.ch, cl = wc.cl, li_h = wc.li_h, li_m = wc.li_m, li_l = wc.li_l;
-    const ExpConsts k = wc.k;
-    double S = 0, s1 = 0, s2 = 0;
-    float Sh = 0, Sl = 0, ah1 = 0, al1 = 0, ah2 = 0, al2 = 0;
-    int cnt = 0;
-    for (long long t = threadIdx.x; t < T; t += kPartialThreads) {
-        const float xv = x[t];
-        float dh, dl;
-        two_sum_f(xv, -xref, dh, dl);  // x - x_ref exactly
-        float ah = ch * dh;
-        float al = fmaf(ch, dh, -ah) + (ch * dl + cl * dh);
-        fast_two_sum_f(ah, al, ah, al);
-        float eh, el;
-        exp_ff(ah, al, k, tab_hi, tab_lo, eh, el);
-        ff_add(Sh, Sl, eh, el);
-        // d = x - lambda_i: x - li_h exactly, then the rest of lambda_i
-        float qh, ql;
-        two_sum_f(xv, -li_h, qh, ql);
-        ff_add(qh, ql, -li_m, -li_l);
-        ff_add(ah1, al1, qh, ql);
-        const float ph = qh * qh;
-        const float pl = fmaf(qh, qh, -ph) + 2.f * qh * ql;
-        ff_add(ah2, al2, ph, pl);
-        if (++cnt == kFlushSamples) {
-            S += (double)Sh + (double)Sl;
-            s1 += (double)ah1 + (double)al1;
-            s2 += (double)ah2 + (double)al2;
-            Sh = Sl = ah1 = al1 = ah2 = al2 = 0.f;
-            cnt = 0;
+    const int r0 = blockIdx.y * per, r1 = min(R, r0 + per);
+    for (int rb = r0; rb < r1; rb += kTeams) {
+        const int r = rb + team;
+        const bool live = r < r1;
+        const float *x = L.x + off + (long long)r * T;
+        float mx = -INFINITY;
+        if (live) {
+#pragma unroll 8
+            for (long long t = tid; t < T; t += kTeamThreads) mx = fmaxf(mx, sgn * x[t]);
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (G > 1 && lane == 0) red_max[warp] = mx;
+        if (G > 1 || rb == r0) __syncthreads();  // the constants and the table are there, and the team's maxima
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (G > 1) mx = fmaxf(mx, red_max[team * G + g]);
+        const float xref = sgn * mx;
+        const float ch = wc.ch, cl = wc.cl, li_h = wc.li;
+        double S = 0, s1 = 0, s2 = 0;
+        if (live) {
+            // blocks of kFlushSamples; the flush stands outside the sample
+            // loop so that its FP64 operations are not speculated per sample
+            // (they were: 87 % of the FP64 pipe, 802 us for 64 x 512 x 1801)
+            for (long long tb = tid; tb < T; tb += (long long)kFlushSamples * kTeamThreads) {
+                float Sh = 0, Sl = 0, ah1 = 0, al1 = 0, ah2 = 0, al2 = 0;
+                const long long te = min(T, tb + (long long)kFlushSamples * kTeamThreads);
+#pragma unroll 4
+                for (long long t = tb; t < te; t += kTeamThreads) {
+                    const float xv = x[t];
+                    float dh, dl;
+                    two_sum_f(xv, -xref, dh, dl);  // x - x_ref exactly
+                    float ah = ch * dh;
+                    float al = fmaf(ch, dh, -ah) + (ch * dl + cl * dh);
+                    fast_two_sum_f(ah, al, ah, al);
+                    float eh, el;
+                    exp_ff(ah, al, tab, tab_hi, tab_lo, eh, el);
+                    ff_sum(Sh, Sl, eh, el);
+                    float qh, ql;
+                    two_sum_f(xv, -li_h, qh, ql);
+                    ff_sum(ah1, al1, qh, ql);
+                    const float ph = qh * qh;
+                    ff_sum(ah2, al2, ph, fmaf(qh, qh, -ph) + 2.f * qh * ql);
+                }
+                S += widen(Sh);
+                s1 += widen(ah1);
+                s2 += widen(ah2);
+                S += widen(Sl);
+                s1 += widen(al1);
+                s2 += widen(al2);
+            }
+        }
+        double v = warp_sum3(S, s1, s2, lane);
+        if (G > 1) {
+            if ((lane & 7) == 0 && lane < 24) red[warp][lane >> 3] = v;
+            __syncthreads();
+            if (tid < 32) {
+                const int q = lane >> 3;  // lanes 0, 8, 16: the three totals
+                if (q < 3)
+#pragma unroll
+                    for (int g = 1; g < G; ++g) v += red[warp + g][q];
+            }
+        }
+        if (live && tid < 32) {
+            const double n = (double)T;
+            const double a1 = __shfl_sync(0xffffffffu, v, 8), a2 = __shfl_sync(0xffffffffu, v, 16);
+            // sums of (x - lambda_i) and its square from those of q = x - lambda_i + lo
+            if (lane == 0)
+                out[(size_t)w * R + r] =
+                    T == 0 ? Partial{INFINITY, 0.0, 0.0, 0.0, 0.0}
+                           : Partial{wc.hkd * (wc.ssum - 2.0 * (double)xref), v, n, a1 - n * wc.lo,
+                                     a2 - wc.lo * (2.0 * a1 - n * wc.lo)};
+        }
+        if (G > 1 && rb + kTeams < r1) __syncthreads();  // red_max and red are free again
     }
-    S += (double)Sh + (double)Sl;
-    s1 += (double)ah1 + (double)al1;
-    s2 += (double)ah2 + (double)al2;
-    const double Sb = block_sum<kPartialThreads>(S, red);
-    const double sdx = block_sum<kPartialThreads>(s1, red);
-    const double sdx2 = block_sum<kPartialThreads>(s2, red);
-    // the minimum of w, taken at x_ref, in the FP64 form of Eq. (9)
-    if (threadIdx.x == 0)
-        out[(size_t)w * L.replicas + r] = Partial{wc.hkd * (wc.ssum - 2.0 * (double)xref), Sb, (double)T, sdx, sdx2};
 }
 
 constexpr int kWindowThreads = 256;
 
 // Replica counts up to this keep the per-replica exponential sums E[r] in
-// shared memory; larger ones recompute them in the jackknife loops.
+// shared memory; larger ones recompute them in the jackknife loop.
 constexpr int kWindowSmemReplicas = 16384;
 
 // Error-free sum of two doubles: s + e == a + b exactly (Knuth's TwoSum).
@@ -346,158 +441,280 @@ __device__ __forceinline__ double sum_without(double hi, double lo, double e_r)
     return v > 0.0 ? v : 0.0;
 }
 
-template <bool SMEM>
-__global__ void __launch_bounds__(kWindowThreads) window_kernel(const ReduceLayout L, const Partial *P, WindowOut *wo)
+// Sum over the warps of half a CTA of a value that each warp holds in the lanes
+// of slot q (lane / width); every thread of the half gets all of them.
+constexpr int kHalf = kWindowThreads / 2, kHalfWarps = kHalf / 32;
+
+__device__ __forceinline__ void half_sync(int half) { asm volatile("bar.sync %0, %1;" ::"r"(1 + half), "r"(kHalf) : "memory"); }
+
+struct CombineArgs {
+    const Partial *P;
+    WindowOut *wo;
+    double *out;
+    unsigned *counter;       // windows finished; 0 between launches (atomicInc wraps)
+    double beta_h, beta_l;   // 1 / kT
+    double k_beta, half_beta2;  // k / kT, 1 / (2 kT^2)
+    double jk, inv_r;        // (R - 1) / R, 1 / R
+    int log2_r;              // ceil(log2 R)
+};
+
+// The profiles are prefix sums over the windows of the per-window increments
+// (and a prefix minimum of the sample counts).  One warp per quantity: a lane
+// adds up s / 32 consecutive windows, the lanes' totals are scanned, and the
+// lane writes its windows' values; the warps' chains run side by side.
+__device__ void profile(const ReduceLayout &L, const CombineArgs &A)
 {
-    extern __shared__ double E[];  // [replicas] when SMEM
-    __shared__ double red[2 * (kWindowThreads / 32 + 1)];
-    const int w = blockIdx.x, R = L.replicas;
-    const Partial *p = P + (size_t)w * R;
-    const double li = L.lambda[w];
-    const double ln = (w + 1 < L.n_windows) ? L.lambda[w + 1] : li;
-    const double d = ln - li;
-    double m = INFINITY;
-    for (int r = threadIdx.x; r < R; r += kWindowThreads)
-        if (p[r].n > 0) m = fmin(m, p[r].m);
-    m = block_min<kWindowThreads>(m, red);
-    // replica r's exponential sum brought to the window's common shift m
-    auto e_of = [&](int r) { return p[r].n > 0 ? p[r].S * exp(-(p[r].m - m) / L.kT) : 0.0; };
-    double se = 0, ce = 0, sn = 0, s1 = 0, c1 = 0, s2 = 0, c2 = 0;
-    for (int r = threadIdx.x; r < R; r += kWindowThreads) {
-        const double e = e_of(r);
-        if (SMEM) E[r] = e;
-        neumaier(se, ce, e);
-        sn += p[r].n;
-        neumaier(s1, c1, p[r].sdx);
-        neumaier(s2, c2, p[r].sdx2);
-    }
-    double Shi, Slo;
-    block_sum_pair<kWindowThreads>(se, ce, red, Shi, Slo);
-    const double S = Shi + Slo;
-    const double n = block_sum<kWindowThreads>(sn, red);
-    const double sdx = block_sum<kWindowThreads>(s1 + c1, red);
-    const double sdx2 = block_sum<kWindowThreads>(s2 + c2, red);
-    const double je = m - L.kT * log(S / n);
-    const double mdx = sdx / n;
-    const double mean = li + mdx;
-    const double var = sdx2 / n - mdx * mdx;
-    const double fl = -L.k * d * mdx;
-    const double g2 = L.k * var / L.kT;
-    // delete-one-replica jackknife, O(R): the leave-one-out exponential sum
-    // from the compensated total (sum_without), the Eq. (14) mean from sdx
-    double vje = 0, vfl = 0;
-    const bool jk = R >= 2;
-    if (jk) {
-        for (int r = threadIdx.x; r < R; r += kWindowThreads) {
-            const double sm = sum_without(Shi, Slo, SMEM ? E[r] : e_of(r));
-            const double nm = n - p[r].n;
-            vje += m - L.kT * log(sm / nm);
-            vfl += -L.k * d * (sdx - p[r].sdx) / nm;
+    const int s = L.n_windows, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = (s + 31) / 32, j0 = lane * k, j1 = min(s, j0 + k);
+    const double *wo = reinterpret_cast<const double *>(A.wo);
+    constexpr int kFields = sizeof(WindowOut) / sizeof(double);
+    auto field = [&](int j, int f) { return __ldcg(wo + (size_t)j * kFields + f); };
+    auto col = [&](int f) { return A.out + (size_t)f * s; };
+    // the lane's exclusive prefix of the other lanes' windows, field f
+    auto before = [&](int f) {
+        double own = 0.0;
+        for (int j = j0; j < j1; ++j)
+            if (j > 0) own += field(j - 1, f);
+        double pre = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, pre, o);
+            if (lane >= o) pre += u;
         }
-    }
-    const double mje = block_sum<kWindowThreads>(vje, red) / R;
-    const double mfl = block_sum<kWindowThreads>(vfl, red) / R;
-    double qje = 0, qfl = 0;
-    if (jk) {
-        for (int r = threadIdx.x; r < R; r += kWindowThreads) {
-            const double sm = sum_without(Shi, Slo, SMEM ? E[r] : e_of(r));
-            const double nm = n - p[r].n;
-            const double a = m - L.kT * log(sm / nm) - mje;
-            const double b = -L.k * d * (sdx - p[r].sdx) / nm - mfl;
-            qje += a * a;
-            qfl += b * b;
+        pre = __shfl_up_sync(0xffffffffu, pre, 1);
+        return lane == 0 ? 0.0 : pre;
+    };
+    // inclusive prefix of field f from the point after lambda_1, fn(j, value)
+    auto scan = [&](int f, auto fn) {
+        double run = before(f);
+        for (int j = j0; j < j1; ++j) {
+            if (j > 0) run += field(j - 1, f);
+            fn(j, run);
         }
+    };
+    enum { kJe, kFl, kG, kWMean, kVarW, kN, kJkJe, kJkFl, kMean, kVar };  // order of WindowOut
+    static_assert(offsetof(WindowOut, mean) == kMean * sizeof(double) && offsetof(WindowOut, jk_je) == kJkJe * sizeof(double),
+                  "WindowOut order");
+    switch (warp) {
+    case 0: {
+        double fl = before(kFl);
+        scan(kJe, [&](int j, double je) {
+            if (j > 0) fl += field(j - 1, kFl);
+            col(kResJE)[j] = je;
+            col(kResCom)[j] = 0.5 * (je + fl);
+            col(kResUnc)[j] = 0.5 * (je - fl);
+        });
+        break;
     }
-    const double sje = block_sum<kWindowThreads>(qje, red);
-    const double sfl = block_sum<kWindowThreads>(qfl, red);
-    if (threadIdx.x == 0) {
-        WindowOut o;
-        o.je = je;
-        o.fl = fl;
-        o.g = L.k * d * d / 2.0 * (1.0 - g2) + fl;
-        o.wmean = 0.5 * L.k * d * (ln + li - 2.0 * mean);
-        o.varw = L.k * L.k * d * d * var;
-        o.n = n;
-        o.jk_je = jk ? (R - 1.0) / R * sje : NAN;
-        o.jk_fl = jk ? (R - 1.0) / R * sfl : NAN;
-        o.mean = mean;
-        o.var = var;
-        wo[w] = o;
+    case 1:
+        scan(kFl, [&](int j, double v) {
+            col(kResFluct)[j] = v;
+            col(kResAccForce)[j] = j > 0 ? v / (L.lambda[j] - L.lambda[0]) : 0.0;
+        });
+        break;
+    case 2: scan(kG, [&](int j, double v) { col(kResG)[j] = v; }); break;
+    case 3: scan(kWMean, [&](int j, double v) { col(kResWMean)[j] = v; }); break;
+    case 4: scan(kJkJe, [&](int j, double v) { col(kResSeJE)[j] = j > 0 ? sqrt(v) : 0.0; }); break;
+    case 5: scan(kJkFl, [&](int j, double v) { col(kResSeFluct)[j] = j > 0 ? sqrt(v) : 0.0; }); break;
+    case 6: {
+        double q = INFINITY;  // smallest sample count of the windows before
+        for (int j = j0; j < j1; ++j)
+            if (j > 0) q = fmin(q, field(j - 1, kN));
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, q, o);
+            if (lane >= o) q = fmin(q, u);
+        }
+        double Q = __shfl_up_sync(0xffffffffu, q, 1);
+        if (lane == 0) Q = INFINITY;
+        scan(kVarW, [&](int j, double v) {
+            if (j > 0) Q = fmin(Q, field(j - 1, kN));
+            // v / Q + v^2 / (2 kT^2 (Q - 1)) over the common denominator
+            const double Q1 = Q - 1.0;
+            col(kResVarZW)[j] = (j > 0 && Q > 1) ? v * fma(v * A.half_beta2, Q, Q1) / (Q * Q1) : (j > 0 ? NAN : 0.0);
+        });
+        break;
+    }
+    default:
+        for (int j = lane; j < s; j += 32) {
+            const double var = field(j, kVar);
+            col(kResLambda)[j] = L.lambda[j];
+            col(kResMeanX)[j] = field(j, kMean);
+            col(kResVarX)[j] = var;
+            col(kResGamma2)[j] = A.k_beta * var;
+        }
     }
 }
 
-// Stage 3: the profiles are prefix sums over the windows of the per-window
-// increments (and a prefix minimum of the sample counts); one CTA scans them
-// kProfileThreads windows at a time (warp shuffles, then the warps' totals),
-// carrying the running totals from one chunk to the next, and every thread
-// writes its window's fields.
-constexpr int kProfileThreads = 256;
-constexpr int kProfileSums = 7;  // je, fl, g, wmean, jk_je, jk_fl, varw
-
-__global__ void __launch_bounds__(kProfileThreads) profile_kernel(const ReduceLayout L, const WindowOut *wo,
-                                                                  double *out)
+// One CTA per window, in two halves that work side by side: warps 0 - 3 on the
+// exponential sums, 4 - 7 on the moments.  The compensated total of the
+// exponential sums comes from an exact split instead of a tree of TwoSums:
+// every e_r is cut at a common bit (adding and subtracting 1.5 2^K, 2^K >= 2 R
+// max e), the upper parts add up without rounding, the lower ones to
+// 2^-106 of the total.  The jackknife's sums are taken about the full estimate,
+// which lies between the leave-one-out values, so one pass serves mean and
+// spread.  The last CTA to finish turns the windows into the profiles.
+template <bool SMEM>
+__global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLayout L, const CombineArgs A)
 {
-    __shared__ double wsum[kProfileThreads / 32][kProfileSums + 1];
-    __shared__ double carry[kProfileSums + 1];
-    const int s = L.n_windows, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid <= kProfileSums) carry[tid] = tid < kProfileSums ? 0.0 : INFINITY;
-    __syncthreads();
-    for (int base = 0; base < s; base += kProfileThreads) {
-        const int j = base + tid;
-        // window j's own terms: the increment of the pair (j - 1, j)
-        double v[kProfileSums + 1];
-        if (j > 0 && j < s) {
-            const WindowOut &o = wo[j - 1];
-            v[0] = o.je; v[1] = o.fl; v[2] = o.g; v[3] = o.wmean; v[4] = o.jk_je; v[5] = o.jk_fl; v[6] = o.varw;
-            v[7] = o.n;
-        } else {
-            for (int q = 0; q < kProfileSums; ++q) v[q] = 0.0;
-            v[kProfileSums] = INFINITY;
-        }
-        // inclusive scan inside the warp
-        for (int o = 1; o < 32; o <<= 1) {
+    extern __shared__ double E[];  // [replicas] when SMEM
+    __shared__ long long red_key[2][kHalfWarps];
+    __shared__ double red[2][kHalfWarps][3], red_q[2][kHalfWarps][2];
+    __shared__ double sh_log;
+    __shared__ int sh_last;
+    const int w = blockIdx.x, R = L.replicas, lane = threadIdx.x & 31;
+    const int half = threadIdx.x >= kHalf, t = threadIdx.x - half * kHalf, hw = t >> 5;
+    const Partial *p = A.P + (size_t)w * R;
+    const bool active = hw * 32 < R;  // the other warps hold no replica and keep off the FP64 unit
+    double m = 0.0;
+    // replica r's exponential sum brought to the window's common shift m
+    auto e_of = [&](int r) {
+        if (!(p[r].n > 0)) return 0.0;
+        const double a = m - p[r].m;
+        return p[r].S * exp(fma(a, A.beta_h, a * A.beta_l));
+    };
+    // max over the half's threads of an integer key
+    auto half_max = [&](long long key, int slot) {
 #pragma unroll
-            for (int q = 0; q <= kProfileSums; ++q) {
-                const double u = __shfl_up_sync(0xffffffffu, v[q], o);
-                if (lane >= o) v[q] = q < kProfileSums ? v[q] + u : fmin(v[q], u);
+        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+        if (lane == 0) red_key[slot][hw] = key;
+        half_sync(0);
+#pragma unroll
+        for (int g = 0; g < kHalfWarps; ++g) key = max(key, red_key[slot][g]);
+        return key;
+    };
+    if (half == 0) {
+        long long key = order_key(-INFINITY);
+        for (int r = t; r < R; r += kHalf)
+            if (p[r].n > 0) key = max(key, order_key(-p[r].m));
+        m = -from_order_key(half_max(key, 0));
+        double e0 = 0.0;  // this thread's first term
+        long long emax = 0;
+        for (int r = t; r < R; r += kHalf) {
+            const double e = e_of(r);
+            if (r == t) e0 = e;
+            if (SMEM) E[r] = e;
+            emax = max(emax, __double_as_longlong(e));
+        }
+        emax = half_max(emax, 1);
+        if (active) {
+            // 1.5 2^K with 2^K >= 2 R max e (NaN and overflowing terms end up in the sums either way)
+            const int K = min(max((int)(emax >> 52) - 1023 + 2 + A.log2_r, -1022), 1023);
+            const double cut = __hiloint2double(((K + 1023) << 20) | 0x80000, 0);
+            double hi = 0.0, lo = 0.0;
+            for (int r = t; r < R; r += kHalf) {
+                const double e = r == t ? e0 : (SMEM ? E[r] : e_of(r));
+                const double u = (e + cut) - cut;
+                hi += u;
+                lo += e - u;
+            }
+            const double v = warp_sum2(hi, lo, lane);
+            if ((lane & 15) == 0) red[0][hw][lane >> 4] = v;
+        }
+    } else if (active) {
+        double sn = 0, s1 = 0, c1 = 0, s2 = 0, c2 = 0;
+        for (int r = t; r < R; r += kHalf) {
+            if (r == t) {
+                sn = p[r].n;
+                s1 = p[r].sdx;
+                s2 = p[r].sdx2;
+            } else {
+                sn += p[r].n;
+                neumaier(s1, c1, p[r].sdx);
+                neumaier(s2, c2, p[r].sdx2);
             }
         }
-        if (lane == 31)
-            for (int q = 0; q <= kProfileSums; ++q) wsum[warp][q] = v[q];
-        __syncthreads();
-        // add the earlier warps' totals and the carry of the earlier chunks
-        double pre[kProfileSums + 1];
-        for (int q = 0; q <= kProfileSums; ++q) pre[q] = carry[q];
-        for (int w = 0; w < warp; ++w)
-            for (int q = 0; q <= kProfileSums; ++q)
-                pre[q] = q < kProfileSums ? pre[q] + wsum[w][q] : fmin(pre[q], wsum[w][q]);
-        for (int q = 0; q <= kProfileSums; ++q) v[q] = q < kProfileSums ? pre[q] + v[q] : fmin(pre[q], v[q]);
-        if (j < s) {
-            double *f[kResFields];
-            for (int q = 0; q < kResFields; ++q) f[q] = out + (size_t)q * s;
-            const double je = v[0], fl = v[1], Q = v[7];
-            const double lam = L.lambda[j];
-            f[kResLambda][j] = lam;
-            f[kResJE][j] = je;
-            f[kResFluct][j] = fl;
-            f[kResG][j] = v[2];
-            f[kResCom][j] = 0.5 * (je + fl);
-            f[kResUnc][j] = 0.5 * (je - fl);
-            f[kResSeJE][j] = j > 0 ? sqrt(v[4]) : 0.0;
-            f[kResSeFluct][j] = j > 0 ? sqrt(v[5]) : 0.0;
-            f[kResVarZW][j] = (j > 0 && Q > 1) ? v[6] / Q + v[6] * v[6] / (2.0 * L.kT * L.kT * (Q - 1.0))
-                                               : (j > 0 ? NAN : 0.0);
-            f[kResWMean][j] = v[3];
-            f[kResAccForce][j] = j > 0 ? fl / (lam - L.lambda[0]) : 0.0;
-            f[kResMeanX][j] = wo[j].mean;
-            f[kResVarX][j] = wo[j].var;
-            f[kResGamma2][j] = L.k * wo[j].var / L.kT;
+        if (R > kHalf) {
+            s1 += c1;
+            s2 += c2;
         }
-        __syncthreads();  // every thread has read carry and wsum
-        if (tid == kProfileThreads - 1)
-            for (int q = 0; q <= kProfileSums; ++q) carry[q] = v[q];
-        __syncthreads();
+        const double v = warp_sum3(sn, s1, s2, lane);
+        if ((lane & 7) == 0 && lane < 24) red[1][hw][lane >> 3] = v;
     }
+    __syncthreads();
+    auto total = [&](int h, int q) {
+        double v = red[h][0][q];
+#pragma unroll
+        for (int g = 1; g < kHalfWarps; ++g)
+            if (g * 32 < R) v += red[h][g][q];
+        return v;
+    };
+    const bool jk = R >= 2, closing = hw == kHalfWarps - 1;  // each half's last warp: the window's own values
+    double q1 = 0, q2 = 0;  // jackknife: sums of the leave-one-out values minus the full estimate, and of their squares
+    double lf = 0.0;
+    if (half == 0) {
+        double Shi = 0, Slo = 0, n = 0;
+        if (active || closing) {
+            const double th = total(0, 0), tl = total(0, 1);
+            n = total(1, 0);
+            Shi = th + tl;
+            Slo = tl - (Shi - th);
+        }
+        auto log_without = [&](int r) {
+            return log(sum_without(Shi, Slo, SMEM ? E[r] : e_of(r)) / (n - p[r].n));
+        };
+        if (closing && lane == 0) sh_log = log((Shi + Slo) / n);  // beside the leave-one-out logarithms
+        double l0 = 0.0;
+        if (jk && t < R) l0 = log_without(t);
+        half_sync(0);
+        lf = sh_log;
+        if (jk)
+            for (int r = t; r < R; r += kHalf) {
+                const double v = L.kT * (lf - (r == t ? l0 : log_without(r)));
+                q1 += v;
+                q2 += v * v;
+            }
+    } else if (active || closing) {
+        const double li = L.lambda[w], ln = w + 1 < L.n_windows ? L.lambda[w + 1] : li, d = ln - li;
+        const double n = total(1, 0), sdx = total(1, 1), kd = -L.k * d;
+        const double mdx = sdx / n;
+        const double fl = kd * mdx;
+        if (jk)
+            for (int r = t; r < R; r += kHalf) {
+                const double v = kd * (sdx - p[r].sdx) / (n - p[r].n) - fl;
+                q1 += v;
+                q2 += v * v;
+            }
+        if (closing && lane == 0) {
+            const double mean = li + mdx, var = total(1, 2) / n - mdx * mdx;
+            WindowOut &o = A.wo[w];
+            o.fl = fl;
+            o.g = L.k * d * d / 2.0 * (1.0 - A.k_beta * var) + fl;
+            o.wmean = 0.5 * L.k * d * (ln + li - 2.0 * mean);
+            o.varw = L.k * L.k * d * d * var;
+            o.n = n;
+            o.mean = mean;
+            o.var = var;
+        }
+    }
+    if (active) {
+        const double v = warp_sum2(q1, q2, lane);
+        if ((lane & 15) == 0) red_q[half][hw][lane >> 4] = v;
+    }
+    half_sync(half);
+    if (t == 0) {
+        double a = red_q[half][0][0], b = red_q[half][0][1];
+#pragma unroll
+        for (int h = 1; h < kHalfWarps; ++h)
+            if (h * 32 < R) {
+                a += red_q[half][h][0];
+                b += red_q[half][h][1];
+            }
+        const double spread = jk ? A.jk * fmax(b - a * a * A.inv_r, 0.0) : NAN;
+        if (half == 0) {
+            A.wo[w].je = m - L.kT * lf;
+            A.wo[w].jk_je = spread;
+        } else {
+            A.wo[w].jk_fl = spread;
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) sh_last = atomicInc(A.counter, (unsigned)L.n_windows - 1) == (unsigned)L.n_windows - 1;
+    __syncthreads();
+    if (!sh_last) return;
+    __threadfence();
+    profile(L, A);
 }
 
 // ---------------------------------------------------------------------------
@@ -619,34 +836,72 @@ cudaError_t state_launch(const ReduceLayout &L, void *scratch, void *turn_partia
     return cudaGetLastError();
 }
 
+constexpr size_t kCounterBytes = 256;
+
 size_t reduce_scratch_bytes(int n_windows, int replicas)
 {
-    return sizeof(Partial) * (size_t)n_windows * replicas + sizeof(WindowOut) * (size_t)n_windows + 256;
+    return sizeof(Partial) * (size_t)n_windows * replicas + sizeof(WindowOut) * (size_t)n_windows + kCounterBytes;
+}
+
+unsigned *reduce_counter(void *buffer, size_t bytes)
+{
+    return reinterpret_cast<unsigned *>(static_cast<char *>(buffer) + bytes - kCounterBytes);
 }
 
 cudaError_t partials_launch(const ReduceLayout &L, void *P, cudaStream_t st)
 {
-    partial_kernel<<<dim3(L.n_windows, L.replicas), kPartialThreads, 0, st>>>(L, static_cast<Partial *>(P));
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // Warps per replica: as few as keep 24 warps on every SM, but no more
+    // than leave a thread four samples.  Replicas per CTA: one turn of its
+    // teams, more where that is more CTAs than fit at once (8 per SM), so that
+    // the window's constants are set less often.
+    // 24 or 16 warps: 30.7, 32.8 us for 21 x 32 x 3600 samples.
+    const long long n = (long long)L.n_windows * L.replicas;
+    int G = 1;
+    while (G < 8 && n * G < 24LL * sms && 64 * G * 4 <= L.t_max) G *= 2;
+    const int teams = kPartialThreads / 32 / G;
+    const long long turns = std::min(8LL, std::max(1LL, n / ((long long)teams * 8 * sms)));
+    const int per = teams * (int)turns;
+    const dim3 grid(L.n_windows, (L.replicas + per - 1) / per);
+    Partial *out = static_cast<Partial *>(P);
+    const ExpTable &tab = exp_table();
+    if (G == 1) partial_kernel<1><<<grid, kPartialThreads, 0, st>>>(L, tab, per, out);
+    else if (G == 2) partial_kernel<2><<<grid, kPartialThreads, 0, st>>>(L, tab, per, out);
+    else if (G == 4) partial_kernel<4><<<grid, kPartialThreads, 0, st>>>(L, tab, per, out);
+    else partial_kernel<8><<<grid, kPartialThreads, 0, st>>>(L, tab, per, out);
     return cudaGetLastError();
 }
 
 cudaError_t combine_launch(const ReduceLayout &L, const void *P, void *window_scratch, double *out, cudaStream_t st)
 {
-    const Partial *pp = static_cast<const Partial *>(P);
-    WindowOut *wo = static_cast<WindowOut *>(window_scratch);
-    cudaError_t e;
+    if (L.counter == nullptr) return cudaErrorInvalidValue;
+    CombineArgs A;
+    A.P = static_cast<const Partial *>(P);
+    A.wo = static_cast<WindowOut *>(window_scratch);
+    A.out = out;
+    A.counter = L.counter;
+    A.beta_h = 1.0 / L.kT;
+    A.beta_l = -std::fma(A.beta_h, L.kT, -1.0) * A.beta_h;
+    A.k_beta = L.k / L.kT;
+    A.half_beta2 = 1.0 / (2.0 * L.kT * L.kT);
+    A.inv_r = 1.0 / L.replicas;
+    A.jk = (L.replicas - 1.0) / L.replicas;
+    A.log2_r = 0;
+    while ((1LL << A.log2_r) < L.replicas) ++A.log2_r;
     if (L.replicas <= kWindowSmemReplicas) {
         const size_t smem = sizeof(double) * (size_t)L.replicas;
-        if (smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(window_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 40 * 1024) {
+            cudaError_t e =
+                cudaFuncSetAttribute(combine_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        window_kernel<true><<<L.n_windows, kWindowThreads, smem, st>>>(L, pp, wo);
+        combine_kernel<true><<<L.n_windows, kWindowThreads, smem, st>>>(L, A);
     } else {
-        window_kernel<false><<<L.n_windows, kWindowThreads, 0, st>>>(L, pp, wo);
+        combine_kernel<false><<<L.n_windows, kWindowThreads, 0, st>>>(L, A);
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    profile_kernel<<<1, kProfileThreads, 0, st>>>(L, wo, out);
     return cudaGetLastError();
 }
 
@@ -751,16 +1006,16 @@ cudaError_t work_samples_launch(const ReduceLayout &L, int mode, long long sampl
 // cudaMalloc.  Every GPU that loads the library holds this array until the
 // process exits, and every call on that GPU reuses it: two calls whose work
 // overlaps on the GPU (different streams, or a second call before the first
-// has finished) write the same scratch and race.  Nothing in it has to start
-// at zero: each call rewrites every entry it later reads.
+// has finished) write the same scratch and race.  Only the counter of
+// finished windows has to start at zero: it does when the module is loaded, and
+// every call leaves it so; each call rewrites every other entry it later reads.
 // ---------------------------------------------------------------------------
 
 namespace {
 
 constexpr size_t kNoAllocPartialBytes = sizeof(Partial) * (size_t)kNoAllocMaxWindowReplicas;
 constexpr size_t kNoAllocWindowBytes = sizeof(WindowOut) * (size_t)kNoAllocMaxWindows;
-constexpr size_t kNoAllocLayoutBytes = 2 * sizeof(long long) * (size_t)kNoAllocMaxWindows;
-constexpr size_t kNoAllocBytes = kNoAllocPartialBytes + kNoAllocWindowBytes + kNoAllocLayoutBytes;
+constexpr size_t kNoAllocBytes = kNoAllocPartialBytes + kNoAllocWindowBytes + kCounterBytes;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -822,15 +1077,6 @@ cudaError_t noalloc_scratch(void **out)
     return cudaSuccess;
 }
 
-__global__ void noalloc_layout_kernel(long long *off, long long *tw, int n_windows, int replicas, long long T)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_windows) {
-        off[i] = (long long)i * replicas * T;
-        tw[i] = T;
-    }
-}
-
 }  // namespace
 
 cudaError_t reduce_noalloc_launch(const float *x, const double *lambda, int n_windows, int replicas,
@@ -840,17 +1086,13 @@ cudaError_t reduce_noalloc_launch(const float *x, const double *lambda, int n_wi
     cudaError_t e = noalloc_scratch(&base);
     if (e != cudaSuccess) return e;
     unsigned char *b = static_cast<unsigned char *>(base);
-    long long *off = reinterpret_cast<long long *>(b + kNoAllocPartialBytes + kNoAllocWindowBytes);
-    long long *tw = off + kNoAllocMaxWindows;
-    noalloc_layout_kernel<<<(n_windows + 127) / 128, 128, 0, st>>>(off, tw, n_windows, replicas, samples_per_window);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     Partial *P = reinterpret_cast<Partial *>(b);
     WindowOut *wo = reinterpret_cast<WindowOut *>(b + kNoAllocPartialBytes);
     ReduceLayout L;
     L.x = x;
     L.lambda = lambda;
-    L.off_w = off;
-    L.tw = tw;
+    L.t_max = samples_per_window;  // no per-window arrays: every window alike
+    L.counter = reduce_counter(base, kNoAllocBytes);
     L.n_windows = n_windows;
     L.replicas = replicas;
     L.k = k;
