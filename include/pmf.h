@@ -433,7 +433,8 @@ pmf_status pmf_chain_set_warps(pmf_system *sys, int chain, int warps);
  * (0: 1000, or an eighth of the launch, at least 16, where that is less and the
  * replicas do not all fit at once) of one replica from a device queue, in segment-major order
  * (ctas = 0 picks: every slot if the replicas fill them, else a whole number
- * of CTAs per SM when that is at least 3, else one CTA per replica); a
+ * of CTAs per SM when that is at least 3, else one CTA per replica; FP64: one
+ * CTA per SM up to 1.7 replicas per SM, else at most two); a
  * replica's next segment waits (at most 60 s, then PMF_ETIMEOUT) until its
  * previous one has stored the state.  Replicas thus migrate between CTAs and
  * no SM idles when the replica count is not a multiple of the SM count.

@@ -44,6 +44,7 @@ template <typename R> struct ChainArgs {
     const Vec2<R> *bead_eq;    // [Np] (sqrt(12 eps), q sqrt(ke)); zero for pads
     const R *bead_invm;        // [Np] 1/m, 0 for pads
     const Vec4<R> *dih;        // [N] (K1 cos d1, K2 cos d2, K3 cos d3, nonzero)
+    const Vec4<R> *pair;       // FP64: pair parameters in ring order (pair_index), (s_ij^2 2^(1/3), 12 eps_ij, k_e q_i q_j, 0)
     Vec4<R> *state;            // [n_rep][2][Np] positions, velocities
     float *xout;               // samples
     const double *lambda;      // [n_windows]
@@ -111,6 +112,8 @@ template <typename R> struct Smem {
     const Vec4<R> *dih;  // [N] dihedral constants
     const int4 *units;   // [NW][max_units] the nonbonded schedule
     const int *ucount;   // [NW]
+    const Vec4<R> *pair; // FP64: pair parameters (global memory)
+    int n_tiles;
     // (shared-memory copies made once per CTA when the chain leaves room for
     // them, else the arguments' global arrays)
     // FP32 packed path: entry p of tile T pairs ring positions p and p + D
@@ -128,7 +131,7 @@ template <typename R> struct Smem {
 // Offset between the two ring steps a packed FP32 double step evaluates.
 __host__ __device__ constexpr int pair_offset(int W) { return W == 32 ? 8 : W / 2; }
 
-__device__ __forceinline__ int tile_width(int t, int n_tiles, int w_last) { return t == n_tiles - 1 ? w_last : 32; }
+__host__ __device__ __forceinline__ int tile_width(int t, int n_tiles, int w_last) { return t == n_tiles - 1 ? w_last : 32; }
 
 template <typename R> __device__ __forceinline__ V3<R> pos_of(const Smem<R> &s, int b)
 {
@@ -202,6 +205,48 @@ __device__ __forceinline__ R pair_fr(const Vec4<R> &pi, const Vec2<R> &qi, const
     return (g * z + ((qi.y * qj.y) * ri - g)) * ri2;  // -dU/dr / r
 }
 
+// Entry of the FP64 pair table for i-tile I, j-tile J, ring step t, lane.
+__host__ __device__ __forceinline__ size_t pair_index(int I, int J, int n_tiles, int t, int lane)
+{
+    return ((size_t)(I * n_tiles + J) * 32 + t) * 32 + lane;
+}
+
+// FP64: this GPU retires one FP64 operation of a warp every 19 cycles per SM
+// and nothing else comes near binding, so operations are traded for loads:
+// the pair's parameters come from a table (four operations less), and
+// 1/sqrt(r2) from the FP32 reciprocal square root by one cubic step,
+// y (1 + e/2 + 3 e^2/8) with e = 1 - r2 y^2 (relative error 5/16 e^3 < 2^-65):
+// 25 operations a pair instead of 31.  r2 beyond FP32's range takes the
+// library's function.
+__device__ __forceinline__ double rsqrt_fast(double v)
+{
+    const int hi = __double2hiint(v), e = hi >> 20;
+    if (e < 1023 - 120 || e > 1023 + 120) return rsqrt(v);
+    // v truncated to FP32 by its bits (a conversion takes a turn of the FP64 unit), and y back
+    const float f = __int_as_float((int)(((unsigned)(hi - (896 << 20)) << 3) | ((unsigned)__double2loint(v) >> 29)));
+    const int y = __float_as_int(rsqrtf(f));
+    const double y0 = __hiloint2double((y >> 3) + (896 << 20), y << 29);
+    const double h = v * y0;
+    const double d = fma(-h, y0, 1.0);
+    return fma(y0 * d, fma(d, 0.375, 0.5), y0);
+}
+
+__device__ __forceinline__ double pair_fr(const Vec4<double> &pi, const Vec4<double> &pj, const Vec4<double> *par, double &dx,
+                                          double &dy, double &dz)
+{
+    const double2 c0 = __ldg(reinterpret_cast<const double2 *>(par)), c1 = __ldg(reinterpret_cast<const double2 *>(par) + 1);
+    dx = pj.x - pi.x;
+    dy = pj.y - pi.y;
+    dz = pj.z - pi.z;
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double ri = rsqrt_fast(r2);
+    const double ri2 = ri * ri;
+    const double x2 = c0.x * ri2;
+    const double z = x2 * x2 * x2;
+    const double g = c0.y * z;
+    return (g * z + (c1.x * ri - g)) * ri2;
+}
+
 template <typename R, int KIND, bool DUAL>
 __device__ __forceinline__ void ring_piece(const Smem<R> &s, Vec4<R> *fw, int I1, int I2, int J, bool near1,
                                            bool near2, int wI, int lane)
@@ -212,26 +257,19 @@ __device__ __forceinline__ void ring_piece(const Smem<R> &s, Vec4<R> *fw, int I1
     const int lr = lane & (W - 1);
     const bool ion = lane < wI;
     Vec4<R> pi1{R(-1e4), R(-1e4), R(-1e4), R(0)}, pi2{R(-2e4), R(-1e4), R(-1e4), R(0)};
-    Vec2<R> qi1{R(0), R(0)}, qi2{R(0), R(0)};
-    if (ion) {
-        pi1 = s.posd[I1 * 64 + lane];
-        qi1 = s.eqd[I1 * 64 + lane];
-    }
-    if (DUAL) {
-        pi2 = s.posd[I2 * 64 + lane];
-        qi2 = s.eqd[I2 * 64 + lane];
-    }
+    if (ion) pi1 = s.posd[I1 * 64 + lane];
+    if (DUAL) pi2 = s.posd[I2 * 64 + lane];
+    const Vec4<R> *c1 = s.pair + pair_index(I1, J, s.n_tiles, TB, lane);
+    const Vec4<R> *c2 = DUAL ? s.pair + pair_index(I2, J, s.n_tiles, TB, lane) : nullptr;
     R f1x = 0, f1y = 0, f1z = 0, f2x = 0, f2y = 0, f2z = 0, fjx = 0, fjy = 0, fjz = 0;
     const Vec4<R> *pj = s.posd + J * 64 + lr;
-    const Vec2<R> *qj = s.eqd + J * 64 + lr;
     const int src = (lane & ~(W - 1)) | ((lr + 1) & (W - 1));
 #pragma unroll
     for (int k = 0; k < NST; ++k) {
         const int t = TB + k;
         const Vec4<R> pjv = pj[t];
-        const Vec2<R> qjv = qj[t];
         R dx, dy, dz;
-        R fr = pair_fr(pi1, qi1, pjv, qjv, dx, dy, dz);
+        R fr = pair_fr(pi1, pjv, c1 + k * 32, dx, dy, dz);
         if (t < 3 && near1) {
             const int d = I1 * 32 + lane - (J * 32 + ((lr + t) & (W - 1)));
             if (d <= 2 && d >= -2) fr = R(0);
@@ -241,7 +279,7 @@ __device__ __forceinline__ void ring_piece(const Smem<R> &s, Vec4<R> *fw, int I1
         fjx += fr * dx; fjy += fr * dy; fjz += fr * dz;
         if (DUAL) {
             R ex, ey, ez;
-            R gr = pair_fr(pi2, qi2, pjv, qjv, ex, ey, ez);
+            R gr = pair_fr(pi2, pjv, c2 + k * 32, ex, ey, ez);
             if (t < 3 && near2) {
                 const int d = I2 * 32 + lane - (J * 32 + ((lr + t) & (W - 1)));
                 if (d <= 2 && d >= -2) gr = R(0);
@@ -636,7 +674,13 @@ struct Team {
     }
 };
 
-template <typename R, int NW, bool SMD, bool SCALAR>
+// NH > 0 (FP64): warps NW .. NW + NH - 1 are helpers.  They compute the bonded
+// terms while the NW pair warps run the ring pieces, and draw the next step's
+// normals while the pair warps update the positions, so that the FP64 unit
+// always has warps to serve; pieces, their order and the force buffers are
+// those of NH = 0, so the results are too.  (FP32 does not gain: its pair warps
+// are the step, and the helpers' registers cost a CTA per SM.)
+template <typename R, int NW, int NH, bool SMD, bool SCALAR>
 __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R> &s, R lam, long long done,
                                             long long nequil, long long sample_base, bool first, uint32_t uid,
                                             long long rec, const Team &tm)
@@ -644,9 +688,14 @@ __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R>
 // `done` steps), or -1 (records are every `stride` steps after nequil).
 {
     const int tid = tm.tid, warp = tid >> 5, lane = tid & 31;
-    gen_noise<R>(a, s, uid, done, first ? 0 : early_noise_blocks(a.N, a.n_tiles, NW), (3 * a.N + 3) >> 2,
-                 NW * 32 - 1 - tid, NW * 32);
-    for (int t = tid; t < a.N; t += NW * 32) {
+    constexpr int kBonded = (NH > 0 ? NH : NW) * 32;  // threads that own bonded terms
+    const int bt = NH > 0 ? tid - NW * 32 : tid;
+    if (NH == 0)
+        gen_noise<R>(a, s, uid, done, first ? 0 : early_noise_blocks(a.N, a.n_tiles, NW), (3 * a.N + 3) >> 2,
+                     NW * 32 - 1 - tid, NW * 32);
+    else if (first && bt >= 0)
+        gen_noise<R>(a, s, uid, done, 0, (3 * a.N + 3) >> 2, bt, kBonded);
+    for (int t = bt; t < a.N && t >= 0; t += kBonded) {
         const R x = bonded_owner(a, s, t, lam);
         if (t == a.N - 1) {
             if (!(x == x) || x > R(1e30)) *s.flag = 1;
@@ -668,7 +717,7 @@ __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R>
             }
         }
     }
-    if (a.nonbonded) {
+    if (a.nonbonded && (NH == 0 || warp < NW)) {
         Vec4<R> *fw_mine = s.fw + warp * a.Np;
         const int cnt = s.ucount[warp];
         const int4 *u = s.units + warp * a.max_units;
@@ -716,11 +765,12 @@ template <> __device__ __forceinline__ Vec4<double> load_cg<double>(const Vec4<d
 // state record, and goes back to it at the end, so a replica's trajectory
 // does not depend on how its steps are cut into launches or segments.
 // Returns false when the run was aborted (non-finite state).
-template <typename R, int NW, bool SMD, bool SCALAR>
+template <typename R, int NW, int NH, bool SMD, bool SCALAR>
 __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s, int rep, int w, int r,
                                          long long s0, long long s1, long long origin, const Team &tm)
 {
     const uint32_t uid = a.uid_base + (uint32_t)rep;
+    constexpr int kThreads = (NW + NH) * 32;
     const int tid = tm.tid;
     const R lam = (R)a.lambda[w];
     const R hdt = R(0.5) * a.dt;
@@ -729,7 +779,7 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
     Vec4<R> *st = a.state + (size_t)rep * 2 * a.Np;
 
     if (tid == 0) *s.flag = 0;
-    for (int b = tid; b < a.Np; b += NW * 32) {
+    for (int b = tid; b < a.Np; b += kThreads) {
         Vec4<R> p, v{0, 0, 0, 0};
         if (s0 == 0) {
             p = a.bead_pos0[b];
@@ -763,13 +813,13 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
         for (int q = 0; q < NW; ++q) s.fw[q * a.Np + b] = Vec4<R>{0, 0, 0, 0};
         for (int m = 0; m < 4; ++m) s.bslot[m * a.Np + b] = Vec4<R>{0, 0, 0, 0};
     }
-    for (int e = tid; e < a.n_tiles * 64; e += NW * 32) {
+    for (int e = tid; e < a.n_tiles * 64; e += kThreads) {
         const int t = e >> 6, i = e & 63, W = tile_width(t, a.n_tiles, a.w_last);
         if (i < 2 * W) s.eqd[e] = a.bead_eq[t * 32 + (i & (W - 1))];
     }
     tm.sync();
     if constexpr (kPacked<R>) {
-        for (int e = tid; e < a.n_tiles * 64; e += NW * 32) {
+        for (int e = tid; e < a.n_tiles * 64; e += kThreads) {
             const int t = e >> 6, i = e & 63, W = tile_width(t, a.n_tiles, a.w_last), D = pair_offset(W);
             if (i >= 2 * W) continue;
             const Vec4<R> p0 = s.posd[t * 64 + (i & (W - 1))], p1 = s.posd[t * 64 + ((i + D) & (W - 1))];
@@ -797,7 +847,7 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
             rec = rec_q++;
             rec_step += a.stride;
         }
-        force_phase<R, NW, SMD, SCALAR>(a, s, SMD ? (R)smd_lambda(a.lambda[0], a.smd_vdt, step, nequil) : lam, step, nequil,
+        force_phase<R, NW, NH, SMD, SCALAR>(a, s, SMD ? (R)smd_lambda(a.lambda[0], a.smd_vdt, step, nequil) : lam, step, nequil,
                                 sample_base, step == s0, uid, rec, tm);
         tm.sync();
         if (step > s0 && *s.flag) {
@@ -806,7 +856,7 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
         }
         // one warp per 32-bead tile (warp-uniform loop: the packed copy is
         // rebuilt with shuffles by the whole warp)
-        for (int tile = warp; tile < a.n_tiles; tile += NW) {
+        for (int tile = warp; tile < a.n_tiles && (NH == 0 || warp < NW); tile += NW) {
             const int b = tile * 32 + lane;
             V3<R> pnew{R(0), R(0), R(0)};
             R sig = R(0);
@@ -855,14 +905,18 @@ __device__ __forceinline__ bool simulate(const ChainArgs<R> &a, const Smem<R> &s
                 if (step < s1) pack_tile(s, tile, lane, tile_width(tile, a.n_tiles, a.w_last), pnew, sig);
             }
         }
-        if (warp >= a.n_tiles && step + 1 < s1)
+        if (NH > 0) {
+            if (warp >= NW && step + 1 < s1)
+                gen_noise<R>(a, s, uid, step + 1, 0, (3 * a.N + 3) >> 2, tid - NW * 32, NH * 32);
+        } else if (warp >= a.n_tiles && step + 1 < s1) {
             gen_noise<R>(a, s, uid, step + 1, 0, early_noise_blocks(a.N, a.n_tiles, NW), tid - a.n_tiles * 32,
                          (NW - a.n_tiles) * 32);
+        }
         if (step >= s1) break;
         tm.sync();
     }
     tm.sync();
-    for (int b = tid; b < a.Np; b += NW * 32) {
+    for (int b = tid; b < a.Np; b += kThreads) {
         const V3<R> p = pos_of(s, b);
         st[b] = Vec4<R>{p.x, p.y, p.z, R(0)};
         st[a.Np + b] = s.vel[b];
@@ -948,12 +1002,14 @@ __device__ __forceinline__ Smem<R> carve_smem(unsigned char *p, const ChainArgs<
     s.dih = a.dih;
     s.units = a.units;
     s.ucount = a.unit_count;
+    s.pair = a.pair;
+    s.n_tiles = a.n_tiles;
     *tail = p;
     return s;
 }
 
-template <typename R, int NW, int CTAS, bool SMD>
-__global__ void __launch_bounds__(NW * 32, CTAS) chain_kernel(const ChainArgs<R> a)
+template <typename R, int NW, int NH, int CTAS, bool SMD>
+__global__ void __launch_bounds__((NW + NH) * 32, CTAS) chain_kernel(const ChainArgs<R> a)
 // SMD: the constant-velocity pulling variant (a separate instantiation, so
 // the window runs carry none of its per-step work bookkeeping).
 // FP32 with 4 warps: five CTAs per SM fit; 6 and 8 warps trade occupancy for
@@ -967,6 +1023,7 @@ __global__ void __launch_bounds__(NW * 32, CTAS) chain_kernel(const ChainArgs<R>
 //    until segment q - 1 has released its state.  Trajectories are
 //    identical in both modes.
 {
+    constexpr int kThreads = (NW + NH) * 32;
     extern __shared__ __align__(32) unsigned char smem_raw[];
     __shared__ long long s_item;
     unsigned char *tail = nullptr;
@@ -977,9 +1034,9 @@ __global__ void __launch_bounds__(NW * 32, CTAS) chain_kernel(const ChainArgs<R>
         Vec4<R> *dih = reinterpret_cast<Vec4<R> *>(p); p += sizeof(Vec4<R>) * a.N;
         int4 *units = reinterpret_cast<int4 *>(p); p += sizeof(int4) * NW * a.max_units;
         int *ucount = reinterpret_cast<int *>(p);
-        for (int e = threadIdx.x; e < NW * a.max_units; e += NW * 32) units[e] = a.units[e];
-        for (int e = threadIdx.x; e < NW; e += NW * 32) ucount[e] = a.unit_count[e];
-        for (int b = threadIdx.x; b < a.N; b += NW * 32) dih[b] = a.dih[b];
+        for (int e = threadIdx.x; e < NW * a.max_units; e += kThreads) units[e] = a.units[e];
+        for (int e = threadIdx.x; e < NW; e += kThreads) ucount[e] = a.unit_count[e];
+        for (int b = threadIdx.x; b < a.N; b += kThreads) dih[b] = a.dih[b];
         s.dih = dih;
         s.units = units;
         s.ucount = ucount;
@@ -1017,8 +1074,8 @@ __global__ void __launch_bounds__(NW * 32, CTAS) chain_kernel(const ChainArgs<R>
             const long long nsteps = a.nsteps_w[w];
             s1 = s1 < nsteps ? s1 : nsteps;
         }
-        const Team tm{(int)threadIdx.x, 0, NW * 32};
-        if ((s0 < s1 || a.force_out != nullptr) && !simulate<R, NW, SMD, NW == 4 && CTAS == 4>(a, s, rep, w, r, s0, s1, origin, tm)) return;
+        const Team tm{(int)threadIdx.x, 0, kThreads};
+        if ((s0 < s1 || a.force_out != nullptr) && !simulate<R, NW, NH, SMD, NW == 4 && CTAS == 4>(a, s, rep, w, r, s0, s1, origin, tm)) return;
         if (a.persistent) {
             __syncthreads();  // the replica's state record is written
             if (threadIdx.x == 0) {
@@ -1174,6 +1231,7 @@ template <typename R> struct ChainDevice {
     Vec2<R> *eq = nullptr;
     R *invm = nullptr;
     Vec4<R> *dih = nullptr;
+    Vec4<R> *pair = nullptr;  // FP64: the pair table
 };
 
 // 2^(1/6): half widths are stored times this, so that (s_i + s_j)^6 / r^6 is
@@ -1213,7 +1271,26 @@ template <typename R> static cudaError_t upload_chain(const ChainHost &h, const 
     if ((e = cudaMemcpy(d.pos0, pos.data(), sizeof(Vec4<R>) * g.Np, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(d.eq, eq.data(), sizeof(Vec2<R>) * g.Np, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(d.invm, invm.data(), sizeof(R) * g.Np, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    return cudaMemcpy(d.dih, dih.data(), sizeof(Vec4<R>) * g.N, cudaMemcpyHostToDevice);
+    if ((e = cudaMemcpy(d.dih, dih.data(), sizeof(Vec4<R>) * g.N, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if constexpr (!kPacked<R>) {
+        // every i-tile I <= J against every ring step of j-tile J; entries of
+        // pads, and of i-beads beyond a ragged tile, stay zero
+        std::vector<Vec4<R>> pair((size_t)g.n_tiles * g.n_tiles * 1024, Vec4<R>{0, 0, 0, 0});
+        for (int J = 0; J < g.n_tiles; ++J) {
+            const int W = tile_width(J, g.n_tiles, g.w_last);
+            for (int I = 0; I <= J; ++I)
+                for (int t = 0; t < W; ++t)
+                    for (int l = 0; l < 32; ++l) {
+                        const int i = I * 32 + l, j = J * 32 + (((l & (W - 1)) + t) & (W - 1));
+                        if (i >= g.Np || i >= h.N || j >= h.N) continue;
+                        const R sg = pos[i].w + pos[j].w;
+                        pair[pair_index(I, J, g.n_tiles, t, l)] = Vec4<R>{sg * sg, eq[i].x * eq[j].x, eq[i].y * eq[j].y, R(0)};
+                    }
+        }
+        if ((e = cudaMalloc(&d.pair, sizeof(Vec4<R>) * pair.size())) != cudaSuccess) return e;
+        return cudaMemcpy(d.pair, pair.data(), sizeof(Vec4<R>) * pair.size(), cudaMemcpyHostToDevice);
+    }
+    return cudaSuccess;
 }
 
 template <typename R> static void free_chain(ChainDevice<R> &d)
@@ -1222,6 +1299,7 @@ template <typename R> static void free_chain(ChainDevice<R> &d)
     cudaFree(d.eq);
     cudaFree(d.invm);
     cudaFree(d.dih);
+    cudaFree(d.pair);
     d = ChainDevice<R>{};
 }
 
@@ -1351,6 +1429,7 @@ static ChainArgs<R> fill_args(const ChainModel::Impl *m, const ChainDevice<R> &d
     a.bead_eq = d.eq;
     a.bead_invm = d.invm;
     a.dih = d.dih;
+    a.pair = d.pair;
     a.state = reinterpret_cast<Vec4<R> *>(L.state);
     a.xout = L.xout;
     a.lambda = L.lambda;
@@ -1429,7 +1508,7 @@ static int auto_segment(long long steps)
     return (int)(s < 16 ? 16 : (s > 1000 ? 1000 : s));
 }
 
-template <typename R, int NW, int CTAS>
+template <typename R, int NW, int CTAS, int NH = 0>
 static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, const RunLaunch &L, cudaStream_t st)
 {
     if (L.smd_vdt != 0.0 && L.wout == nullptr) return cudaErrorInvalidValue;  // a pulled run records its work
@@ -1437,7 +1516,7 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
     bool extras = false;
     const size_t smem = chain_smem_bytes<R>(m->geo, NW, m->max_units, &extras);
     a.static_in_smem = extras ? 1 : 0;
-    void (*kern)(const ChainArgs<R>) = a.smd ? chain_kernel<R, NW, CTAS, true> : chain_kernel<R, NW, CTAS, false>;
+    void (*kern)(const ChainArgs<R>) = a.smd ? chain_kernel<R, NW, NH, CTAS, true> : chain_kernel<R, NW, NH, CTAS, false>;
     // The attribute is the kernel's upper limit, shared by every chain that
     // launches it: raise it to the device's opt-in maximum rather than to this
     // chain's size, so launches captured earlier in a graph (other chains,
@@ -1460,7 +1539,7 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
         // persistent: as many CTAs as fit at once (or as requested), never
         // more than there are replicas
         int occ = 0, sms = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NW * 32, smem)) !=
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, (NW + NH) * 32, smem)) !=
             cudaSuccess)
             return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -1472,7 +1551,9 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
             // queue ahead of the running segments, so no CTA waits), unless
             // that number is below 3, where more CTAs per SM still pay
             const long long per_sm = L.n_blocks / sms;
-            want = L.n_blocks >= slots ? slots : (per_sm >= 3 ? per_sm * sms : L.n_blocks);
+            if (sizeof(R) == 8) want = NH > 0 ? sms : std::min<long long>(L.n_blocks, 2LL * sms);
+            else
+                want = L.n_blocks >= slots ? slots : (per_sm >= 3 ? per_sm * sms : L.n_blocks);
         }
         grid = (int)std::min<long long>(want, L.n_blocks);
         if (!L.sequential && m->seg_auto && grid < L.n_blocks) a.seg_steps = auto_segment(L.step_end - L.step_begin);
@@ -1483,7 +1564,7 @@ static cudaError_t launch_typed(ChainModel::Impl *m, const ChainDevice<R> &d, co
         if ((e = cudaMemsetAsync(L.queue, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(L.done, 0, sizeof(int) * (size_t)L.n_blocks, st)) != cudaSuccess) return e;
     }
-    kern<<<grid, NW * 32, smem, st>>>(a);
+    kern<<<grid, (NW + NH) * 32, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1553,7 +1634,7 @@ __device__ __forceinline__ bool pack_team(const ChainArgs<R> &a, unsigned char *
 {
     unsigned char *tail = nullptr;
     const Smem<R> s = carve_smem<R, G>(base, a, &tail);
-    return simulate<R, G, false, false>(a, s, rep, rep / a.replicas, rep % a.replicas, s0, s1, 0, tm);
+    return simulate<R, G, 0, false, false>(a, s, rep, rep / a.replicas, rep % a.replicas, s0, s1, 0, tm);
 }
 
 template <typename R>
@@ -1791,6 +1872,15 @@ int pack_plan_packs(const PackPlan *plan) { return plan ? plan->args.n_packs : 0
 int pack_plan_grid(const PackPlan *plan) { return plan ? plan->grid : 0; }
 size_t pack_plan_smem(const PackPlan *plan) { return plan ? plan->smem : 0; }
 
+static int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return std::max(sms, 1);
+}
+
 // Four warps a replica, two builds of the same arithmetic (bit-identical):
 // four CTAs per SM with 128 registers a thread, which lets the compiler
 // overlap the ring steps, or five with 96.  The fifth CTA pays only where
@@ -1799,18 +1889,19 @@ size_t pack_plan_smem(const PackPlan *plan) { return plan ? plan->smem : 0; }
 // 64 11533 / 11371, 72 17455 / 16577, 80 19498 / 19970, 104 24999 / 25923;
 // with 672 replicas four win at every length (40 beads 5739 / 5997, 104
 // 12997 / 13863).
-static bool small_chain_ctas(const ChainGeometry &g, int n_rep)
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return false;
-    return g.Np <= 72 && n_rep >= 5 * sms;
-}
+static bool small_chain_ctas(const ChainGeometry &g, int n_rep) { return g.Np <= 72 && n_rep >= 5 * sm_count(); }
 
 cudaError_t ChainModel::launch(const RunLaunch &L, cudaStream_t st)
 {
-    if (p->precision == 1) return launch_typed<double, 4, 1>(p, p->dd, L, st);
+    if (p->precision == 1) {
+        // FP64: with up to 1.7 replicas per SM one CTA of four pair and four
+        // helper warps on each, the replicas migrating; with more, two CTAs
+        // of four warps (a third only thrashes L1).  104 beads, ms for 96
+        // steps, helpers on 152 / two CTAs per SM / before: 168 replicas 7.8,
+        // 10.1, 12.3; 301: 13.8, 11.9, 19.5; 672: 31.0, 25.4, 34.7
+        if ((long long)L.n_blocks * 10 < 17LL * sm_count()) return launch_typed<double, 4, 1, 4>(p, p->dd, L, st);
+        return launch_typed<double, 4, 1>(p, p->dd, L, st);
+    }
     if (p->NW == 5) return launch_typed<float, 5, 4>(p, p->df, L, st);
     if (p->NW == 6) return launch_typed<float, 6, 3>(p, p->df, L, st);
     if (p->NW == 8) return launch_typed<float, 8, 2>(p, p->df, L, st);

@@ -1,8 +1,9 @@
 """Launch rules of the chain kernel: short default launches cut their steps
 into segments when the replicas do not all fit at once, and short chains with
-many replicas run the five-CTA build.  Neither changes a bit of the result:
-replica (w, r) with uid u equals the same uid in a launch of few replicas
-(every one resident, one segment, the four-CTA build)."""
+many replicas run the five-CTA build; FP64 launches of few replicas have helper
+warps for the bonded terms and the noise.  None of it changes a bit of the
+result: replica (w, r) with uid u equals the same uid in a launch of few
+replicas (every one resident, one segment, the four-CTA build, helpers)."""
 import numpy as np
 import pytest
 
@@ -18,7 +19,7 @@ def pmf():
     return m
 
 
-def _run(pmf, sysh, lam, replicas, n_steps, uid_base=0, prec=0):
+def _run(pmf, sysh, lam, replicas, n_steps, uid_base=0):
     run = inputs.RunSettings(k=500.0, kT=inputs.kT_of(300.0), dt=0.001, gamma=5.0, n_steps=n_steps, n_equil=5,
                              stride=3, replicas=replicas, seed=23)
     rr = pmf.pmf_run_windows(sysh, lam, pmf.make_params(run, uid_base=uid_base))
@@ -27,12 +28,15 @@ def _run(pmf, sysh, lam, replicas, n_steps, uid_base=0, prec=0):
 
 # lengths around the five-CTA line (72 padded beads), one tile to five;
 # steps below, at and off multiples of the shortest segment (16)
+@pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("n,steps", [(13, 40), (40, 16), (72, 33), (73, 17), (104, 50), (130, 35)])
-def test_many_replicas_equal_few(pmf, n, steps):
+def test_many_replicas_equal_few(pmf, n, steps, prec):
     p = inputs.chain_params(n, 40 + n)
     start = f32(inputs.chain_start(p, 50 + n))
     lam = np.array([1.0, 1.2])
-    sysh = pmf.pmf_create_system_chain([p], [start])
+    sysh = pmf.pmf_create_system_chain([p], [start], precision=prec)
+    if prec:
+        steps = min(steps, 20)
     R = 450  # 900 replicas: more than five CTAs on each of 152 SMs
     xm, pm = _run(pmf, sysh, lam, R, steps)
     for w, r0 in ((0, 0), (1, R - 6)):
