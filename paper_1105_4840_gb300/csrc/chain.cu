@@ -674,12 +674,12 @@ struct Team {
     }
 };
 
-// NH > 0 (FP64): warps NW .. NW + NH - 1 are helpers.  They compute the bonded
-// terms while the NW pair warps run the ring pieces, and draw the next step's
-// normals while the pair warps update the positions, so that the FP64 unit
-// always has warps to serve; pieces, their order and the force buffers are
-// those of NH = 0, so the results are too.  (FP32 does not gain: its pair warps
-// are the step, and the helpers' registers cost a CTA per SM.)
+// NH > 0 (few replicas per SM): warps NW .. NW + NH - 1 are helpers.  They compute
+// the bonded terms while the NW pair warps run the ring pieces, and draw the
+// next step's normals while the pair warps update the positions; pieces, their
+// order and the force buffers are those of NH = 0, so the results are too.
+// (With three replicas per SM and more the other CTAs fill those gaps, and the
+// helpers' registers would cost a CTA per SM.)
 template <typename R, int NW, int NH, bool SMD, bool SCALAR>
 __device__ __forceinline__ void force_phase(const ChainArgs<R> &a, const Smem<R> &s, R lam, long long done,
                                             long long nequil, long long sample_base, bool first, uint32_t uid,
@@ -1904,7 +1904,14 @@ cudaError_t ChainModel::launch(const RunLaunch &L, cudaStream_t st)
     }
     if (p->NW == 5) return launch_typed<float, 5, 4>(p, p->df, L, st);
     if (p->NW == 6) return launch_typed<float, 6, 3>(p, p->df, L, st);
+    // eight warps, up to one replica per SM: four helpers (104 beads, 147
+    // replicas: 5594 -> 4797; 333 beads 23706 -> 22336)
+    if (p->NW == 8 && L.n_blocks <= sm_count()) return launch_typed<float, 8, 1, 4>(p, p->df, L, st);
     if (p->NW == 8) return launch_typed<float, 8, 2>(p, p->df, L, st);
+    // up to two replicas per SM: two helper warps and 168 registers a thread
+    // (104 beads, cycles per step: 147 replicas 7137 -> 6085, 301 7849 -> 7216;
+    // 455, three per SM, 9534 -> 11066)
+    if (L.n_blocks <= 2 * sm_count()) return launch_typed<float, 4, 2, 2>(p, p->df, L, st);
     if (small_chain_ctas(p->geo, L.n_blocks)) return launch_typed<float, 4, 5>(p, p->df, L, st);
     return launch_typed<float, 4, 4>(p, p->df, L, st);
 }
