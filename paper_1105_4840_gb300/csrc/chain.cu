@@ -1238,6 +1238,23 @@ template <typename R> struct ChainDevice {
 // z = 2 (s_ij / r)^6 and -dU_LJ/dr r = 12 eps_ij (z^2 - z).
 constexpr double kLjScale = 1.122462048309372981433533;
 
+// The FP64 pair table: every i-tile I <= J against every ring step of j-tile
+// J; entries of pads, and of i-beads beyond a ragged tile, are zero.
+__global__ void pair_table_kernel(const Vec4<double> *pos0, const Vec2<double> *eq, int N, int n_tiles, int w_last,
+                                  Vec4<double> *pair)
+{
+    const size_t at = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (at >= (size_t)n_tiles * n_tiles * 1024) return;
+    const int l = (int)(at & 31), t = (int)((at >> 5) & 31), IJ = (int)(at >> 10), I = IJ / n_tiles, J = IJ % n_tiles;
+    const int W = tile_width(J, n_tiles, w_last), i = I * 32 + l, j = J * 32 + (((l & (W - 1)) + t) & (W - 1));
+    Vec4<double> v{0, 0, 0, 0};
+    if (I <= J && t < W && i < N && j < N && l < tile_width(I, n_tiles, w_last)) {
+        const double sg = pos0[i].w + pos0[j].w;
+        v = Vec4<double>{sg * sg, eq[i].x * eq[j].x, eq[i].y * eq[j].y, 0};
+    }
+    pair[at] = v;
+}
+
 template <typename R> static cudaError_t upload_chain(const ChainHost &h, const ChainGeometry &g, ChainDevice<R> &d)
 {
     std::vector<Vec4<R>> pos(g.Np), dih(g.N);
@@ -1273,22 +1290,11 @@ template <typename R> static cudaError_t upload_chain(const ChainHost &h, const 
     if ((e = cudaMemcpy(d.invm, invm.data(), sizeof(R) * g.Np, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if ((e = cudaMemcpy(d.dih, dih.data(), sizeof(Vec4<R>) * g.N, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
     if constexpr (!kPacked<R>) {
-        // every i-tile I <= J against every ring step of j-tile J; entries of
-        // pads, and of i-beads beyond a ragged tile, stay zero
-        std::vector<Vec4<R>> pair((size_t)g.n_tiles * g.n_tiles * 1024, Vec4<R>{0, 0, 0, 0});
-        for (int J = 0; J < g.n_tiles; ++J) {
-            const int W = tile_width(J, g.n_tiles, g.w_last);
-            for (int I = 0; I <= J; ++I)
-                for (int t = 0; t < W; ++t)
-                    for (int l = 0; l < 32; ++l) {
-                        const int i = I * 32 + l, j = J * 32 + (((l & (W - 1)) + t) & (W - 1));
-                        if (i >= g.Np || i >= h.N || j >= h.N) continue;
-                        const R sg = pos[i].w + pos[j].w;
-                        pair[pair_index(I, J, g.n_tiles, t, l)] = Vec4<R>{sg * sg, eq[i].x * eq[j].x, eq[i].y * eq[j].y, R(0)};
-                    }
-        }
-        if ((e = cudaMalloc(&d.pair, sizeof(Vec4<R>) * pair.size())) != cudaSuccess) return e;
-        return cudaMemcpy(d.pair, pair.data(), sizeof(Vec4<R>) * pair.size(), cudaMemcpyHostToDevice);
+        const size_t n = (size_t)g.n_tiles * g.n_tiles * 1024;
+        if ((e = cudaMalloc(&d.pair, sizeof(Vec4<R>) * n)) != cudaSuccess) return e;
+        pair_table_kernel<<<(unsigned)((n + 255) / 256), 256>>>(d.pos0, d.eq, h.N, g.n_tiles, g.w_last, d.pair);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        return cudaStreamSynchronize(nullptr);
     }
     return cudaSuccess;
 }
