@@ -1219,7 +1219,7 @@ pmf_status pmf_free_energy_from_partials(const double *partials, const double *l
     L.replicas = replicas;
     L.k = k;
     L.kT = kT;
-    cudaError_t e = combine_launch(L, t.P, t.wo, t.res, g_stream);
+    cudaError_t e = combine_launch(L, t.P, t.wo, t.res, g_stream, false);
     if (e != cudaSuccess) return cuda_fail(e, "combine");
     std::vector<double> h((size_t)kResFields * n_windows);
     CK(cudaMemcpyAsync(h.data(), t.res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, g_stream), "copy");

@@ -184,7 +184,7 @@ cudaError_t smd_stats_launch(const double *W, const float *x, int R, long long T
 size_t partial_bytes(int n_windows, int replicas);
 cudaError_t partials_launch(const ReduceLayout &L, void *partials, cudaStream_t st);
 cudaError_t combine_launch(const ReduceLayout &L, const void *partials, void *window_scratch, double *out,
-                           cudaStream_t st);
+                           cudaStream_t st, bool behind_partials);
 // Allocation-free reduction: scratch in a fixed device array, equal samples
 // per window, all pointers on the device.
 constexpr int kNoAllocMaxWindows = 1024;

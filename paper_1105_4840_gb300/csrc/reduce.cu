@@ -302,6 +302,10 @@ __global__ void __launch_bounds__(kPartialThreads, G >= 4 ? 5 : 4) partial_kerne
         wc.li = (float)li;
         wc.lo = li - (double)wc.li;
     }
+    // The combination may be launched meanwhile (its CTAs wait for this grid's
+    // end).  Not with one-warp teams, the rule for grids that fill the chip for
+    // long: 64 x 512 x 1801 samples took 322 us with it, 272 without.
+    if (G > 1) cudaTriggerProgrammaticLaunchCompletion();
     const int r0 = blockIdx.y * per, r1 = min(R, r0 + per);
     for (int rb = r0; rb < r1; rb += kTeams) {
         const int r = rb + team;
@@ -565,6 +569,7 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
     const int w = blockIdx.x, R = L.replicas, lane = threadIdx.x & 31;
     const int half = threadIdx.x >= kHalf, t = threadIdx.x - half * kHalf, hw = t >> 5;
     const Partial *p = A.P + (size_t)w * R;
+    cudaGridDependencySynchronize();  // the partials are there (returns at once after an ordinary launch)
     const bool active = hw * 32 < R;  // the other warps hold no replica and keep off the FP64 unit
     double m = 0.0;
     // replica r's exponential sum brought to the window's common shift m
@@ -875,7 +880,29 @@ cudaError_t partials_launch(const ReduceLayout &L, void *P, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t combine_launch(const ReduceLayout &L, const void *P, void *window_scratch, double *out, cudaStream_t st)
+// behind_partials: the stream's last operation is this call's partials launch,
+// whose tail the combination's launch overlaps (it waits for that grid before it
+// reads): 5 x 4 x 256 samples 20.5 -> 17.3 us, 21 x 32 x 3600 30.7 -> 28.7 us.
+// Behind anything else (gathered partials) an ordinary launch.
+template <typename K>
+static cudaError_t launch_combine(K kernel, size_t smem, bool behind_partials, cudaStream_t st, const ReduceLayout &L,
+                                  const CombineArgs &A)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)L.n_windows);
+    cfg.blockDim = dim3(kWindowThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = behind_partials ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, L, A);
+}
+
+cudaError_t combine_launch(const ReduceLayout &L, const void *P, void *window_scratch, double *out, cudaStream_t st,
+                           bool behind_partials)
 {
     if (L.counter == nullptr) return cudaErrorInvalidValue;
     CombineArgs A;
@@ -898,11 +925,9 @@ cudaError_t combine_launch(const ReduceLayout &L, const void *P, void *window_sc
                 cudaFuncSetAttribute(combine_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        combine_kernel<true><<<L.n_windows, kWindowThreads, smem, st>>>(L, A);
-    } else {
-        combine_kernel<false><<<L.n_windows, kWindowThreads, 0, st>>>(L, A);
+        return launch_combine(combine_kernel<true>, smem, behind_partials, st, L, A);
     }
-    return cudaGetLastError();
+    return launch_combine(combine_kernel<false>, 0, behind_partials, st, L, A);
 }
 
 // Constant-velocity pulling, record j (one block each): over the replicas,
@@ -957,7 +982,7 @@ cudaError_t reduce_launch(const ReduceLayout &L, void *scratch, double *out, cud
     void *wo = static_cast<char *>(scratch) + partial_bytes(L.n_windows, L.replicas);
     cudaError_t e = partials_launch(L, P, st);
     if (e != cudaSuccess) return e;
-    return combine_launch(L, P, wo, out, st);
+    return combine_launch(L, P, wo, out, st, true);
 }
 
 __global__ void work_increment_kernel(const ReduceLayout L, double *out)
@@ -1098,7 +1123,7 @@ cudaError_t reduce_noalloc_launch(const float *x, const double *lambda, int n_wi
     L.k = k;
     L.kT = kT;
     if ((e = partials_launch(L, P, st)) != cudaSuccess) return e;
-    return combine_launch(L, P, wo, out, st);
+    return combine_launch(L, P, wo, out, st, true);
 }
 
 }  // namespace pmf
