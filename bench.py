@@ -144,15 +144,15 @@ def _reduction_roofline(ms, n_samples, peaks, fp64_tflops):
     """The reductions of one step against HBM (4 bytes of x per sample, read
     by each of stage 1's two passes) and beside the measured FP64 rate:
     stage 1 forms its exponentials and per-thread sums in double-float
-    arithmetic on the FP32 pipe; three dependent launches of a few tens of
+    arithmetic on the FP32 pipe; two dependent launches of 10 to 15
     microseconds, not HBM, bound the whole."""
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     gbs = 4.0 * n_samples / (ms * 1e-3) / 1e9
-    return {"kernels": "partial_kernel, window_kernel, profile_kernel", "ms": ms, "samples": n_samples,
+    return {"kernels": "partial_kernel, combine_kernel", "ms": ms, "samples": n_samples,
             "bound": "latency", "achieved_gbs": gbs, "hbm_peak_gbs": hbm, "hbm_frac": gbs / hbm,
             "ns_per_sample": ms * 1e6 / n_samples, "fp64_tflops_measured": fp64_tflops,
-            "note": "stage 1 in double-float arithmetic on the FP32 pipe (FP64 per flush of 16 samples and in the "
-                    "block trees); three dependent launches, not HBM, bound the reduction"}
+            "note": "stage 1 in double-float arithmetic on the FP32 pipe (FP64 per flush of a block of samples and "
+                    "in the last sums); two dependent launches, not HBM, bound the reduction"}
 
 
 def cpu_baseline(budget_s=12.0, n_steps=200, single_thread=True):
@@ -314,7 +314,7 @@ def bench_batch(args, pmf, torch, stream):
                                                                           binfo["policy"], teams))
                        if packed else "one CUDA graph, one branch per chain",
                        "autotune_probe_ms": tune_ms, "l2": "256 MB flush between timed steps"},
-            "gpu_launches": args.steps * (chunks + 3 * len(lams)),
+            "gpu_launches": args.steps * (chunks + 2 * len(lams)),
             "clocks": {"sm_mhz": clk.get("sm_mhz"), "sm_max_mhz": clk.get("sm_max_mhz"),
                        "reasons": clk.get("reasons")},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -636,7 +636,8 @@ def bench_mlp(args, pmf, torch, stream):
     """Surrogate training throughput: Adam steps of the 1 -> 64 -> 64 -> 2
     network (64 x 64 layer on tcgen05, BF16 operands, FP32 accumulators in
     TMEM) on mini-batches drawn from a 1D run's sample store, split (a CTA
-    per 128-sample tile, then an update launch, per step) and in one CTA."""
+    per 128-sample tile, up to 8 as one cluster that runs all steps) and in
+    one CTA."""
     from paper_1105_4840_gb300 import inputs
 
     w = inputs.od1d_workload()
@@ -1110,7 +1111,7 @@ def main():
                        "schedule_variant": pmf.pmf_chain_get_schedule(sysh, 0)},
             "e2e": {"value": e2e_value, "unit": "replica-steps/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},
-            "gpu_launches": args.steps * (chunks + 3),
+            "gpu_launches": args.steps * (chunks + 2),
             "clocks": {"sm_mhz": clk.get("sm_mhz"), "sm_max_mhz": clk.get("sm_max_mhz"),
                        "reasons": clk.get("reasons")},
             "roofline": roof,

@@ -498,13 +498,16 @@ pmf_status pmf_mlp_gradient(pmf_mlp *mlp, const double *lambda, const float *x, 
 pmf_status pmf_mlp_train(pmf_mlp *mlp, const pmf_run *run, int steps, int batch, double lr, uint64_t seed,
                          double *loss);
 /* How training (pmf_mlp_train and the adaptive protocol's rounds) runs on
- * the GPU.  split = 1 (the default): every Adam step is one launch with a
- * CTA per 128-sample tile of the batch, each writing its tile's gradient,
- * then an update launch that sums the tiles in tile order and applies Adam;
- * the scratch ([tiles][PMF_MLP_PARAMS] floats) is allocated on first use and
- * kept with the surrogate.  split = 0: one CTA runs all steps, the tiles of
- * a step one after another.  Both draw the same mini-batches; they differ
- * only in FP32 summation order.  PMF_EINVAL for other values. */
+ * the GPU.  split = 1 (the default): a CTA per 128-sample tile of the batch.
+ * With 2 to 8 tiles (batches of 129 to 1024) they form one cluster that runs
+ * all steps in a launch and exchanges gradients and weights through
+ * distributed shared memory; with more tiles every step is a tile launch and
+ * an update launch that sums the tiles' gradients in tile order and applies
+ * Adam.  The scratch of the latter ([tiles][PMF_MLP_PARAMS] floats) is
+ * allocated on first use and kept with the surrogate.  split = 0: one CTA runs
+ * all steps, the tiles of a step one after another.  All draw the same
+ * mini-batches; the two splits give the same bits, split = 0 differs only in
+ * FP32 summation order.  PMF_EINVAL for other values. */
 pmf_status pmf_mlp_set_split(pmf_mlp *mlp, int split);
 
 /* ---- adaptive protocol: surrogate-guided window insertion -----------------

@@ -21,7 +21,9 @@
 //    buffers (deterministic order), so a run is bit-reproducible;
 //  * bonded terms (bond, angle, three-term dihedral) are computed once by the
 //    thread owning their first bead, written to per-owner slots and gathered;
-//  * BAOAB with Philox4x32-10 noise, counter (bead, uid, step, 0).
+//  * BAOAB with Philox4x32-10 noise, counter (bead, uid, step, 0);
+//  * where a launch leaves warp slots free (few replicas per SM; FP64), helper
+//    warps compute the bonded terms and the noise beside the pair warps.
 #include <algorithm>
 #include <memory>
 #include <cmath>

@@ -219,9 +219,10 @@ struct MlpLaunch {
     float *out_grad = nullptr;
     double *out_loss = nullptr;
     int *err = nullptr;
-    // training (mode 2) with split: one CTA per 128-sample tile and an
-    // update kernel per step; tile_grad [tile_cap][kMlpParams] and
-    // tile_loss [tile_cap] are the caller's scratch
+    // training (mode 2) with split: one CTA per 128-sample tile, up to 8 as a
+    // cluster that runs all steps, more with an update kernel per step;
+    // tile_grad [tile_cap][kMlpParams] and tile_loss [tile_cap] are the caller's
+    // scratch for the latter
     bool split = false;
     float *tile_grad = nullptr;
     double *tile_loss = nullptr;

@@ -863,7 +863,7 @@ cudaError_t partials_launch(const ReduceLayout &L, void *P, cudaStream_t st)
     // than leave a thread four samples.  Replicas per CTA: one turn of its
     // teams, more where that is more CTAs than fit at once (8 per SM), so that
     // the window's constants are set less often.
-    // 24 or 16 warps: 30.7, 32.8 us for 21 x 32 x 3600 samples.
+    // 24 or 16 warps: 30.7, 32.8 us for 21 x 32 x 3600 samples (ordinary launches).
     const long long n = (long long)L.n_windows * L.replicas;
     int G = 1;
     while (G < 8 && n * G < 24LL * sms && 64 * G * 4 <= L.t_max) G *= 2;
