@@ -627,6 +627,12 @@ pmf_status pmf_philox(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint
 pmf_status pmf_chain_forces(pmf_system *sys, int chain, const double *pos, double lambda,
                             double k, double *forces);
 
+/* The records that one of the 1D integrator's three helper warps takes in a
+ * window of n_equil equilibration steps, from step `from` on (host, no GPU
+ * needed): record number at[i] is taken at the end of step step[i], i < n.
+ * PMF_EINVAL for helper outside 0..2, stride < 1 or negative counts. */
+pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t from, int n, int64_t *at, int64_t *step);
+
 /* Overlap coefficients ovl[i] = int min(p_i, p_{i+1}) dx, i < n - 1, of the
  * Gaussians N(mu_i, exp(log_var_i)) (host arrays), computed by the kernel
  * the adaptive protocol uses. */

@@ -2119,6 +2119,19 @@ pmf_status pmf_philox(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint
     return PMF_OK;
 }
 
+pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t from, int n, int64_t *at, int64_t *step)
+{
+    if (helper < 0 || helper >= kOd1dHelpers || n_equil < 0 || stride < 1 || from < 0 || n < 0 || (n > 0 && (!at || !step)))
+        return fail(PMF_EINVAL, "pmf_od1d_records: bad argument");
+    RecordWalk walk;
+    walk.enter(0, n_equil, stride, from, helper);
+    for (int i = 0; i < n; ++i, walk.next(stride)) {
+        at[i] = walk.at;
+        step[i] = walk.rec;
+    }
+    return PMF_OK;
+}
+
 pmf_status pmf_chain_schedule(int N, int NW, int precision, int *out, size_t capacity, size_t *n_written,
                               int *padded)
 {

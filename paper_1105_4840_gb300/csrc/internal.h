@@ -149,6 +149,27 @@ struct Od1dParams {
 // steps; the state holds x and the pulling work per simulation (2 doubles).
 cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cudaStream_t st);
 long long od1d_noise_steps(int n_rep);
+// Records of one window of a 1D simulation that one helper warp of kOd1dHelpers
+// takes (record number `at`: helper at mod kOd1dHelpers).  rec: the step whose end
+// it is taken at; 64 bits throughout: strides go up to 2^31 - 1, step counts
+// to 2^32 - 1.
+constexpr int kOd1dHelpers = 3;
+struct RecordWalk {
+    long long rec = 0, at = 0;
+    // first record of this helper not taken before step `from` of a window whose first step is `origin`
+    __host__ __device__ void enter(long long origin, long long nequil, int stride, long long from, int helper)
+    {
+        const long long past = from - origin - nequil;
+        const long long at0 = past > 0 ? past / stride : 0;
+        at = at0 + (helper + kOd1dHelpers - at0 % kOd1dHelpers) % kOd1dHelpers;
+        rec = origin + nequil + (at + 1) * stride - 1;
+    }
+    __host__ __device__ void next(int stride)
+    {
+        rec += (long long)kOd1dHelpers * stride;
+        at += kOd1dHelpers;
+    }
+};
 
 // FP64 reductions of x samples into the estimators.
 struct ReduceLayout {

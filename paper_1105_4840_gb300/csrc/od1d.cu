@@ -227,20 +227,16 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         if (lane == 0) dbl_mask[b] = mask;
     };
 
-    // warps 1 - 3: the records of a finished tile, record number `at` of a
-    // window by helper at mod 3; no division in the loop.  rec: step whose end
-    // the helper's next record is taken at.
+    // warps 1 - 3: the records of a finished tile; no division in the loop
     const int helper = warp - 1;
-    constexpr int kHelpers = kOd1dThreads / 32 - 1;
+    static_assert(kOd1dHelpers == kOd1dThreads / 32 - 1, "every warp but the first records");
     int ww = w;
-    long long rec = 0, at = 0, base = 0, wend = 0;
+    RecordWalk walk;
+    long long base = 0, wend = 0;
     auto enter_window = [&](int window, long long from) {
         ww = window;
         const long long origin = a.sequential ? (long long)ww * a.window_steps : 0;
-        const long long past = from - origin - a.nequil_w[ww];
-        const long long at0 = past > 0 ? past / a.stride : 0;  // records taken before step `from`
-        at = at0 + (helper + kHelpers - at0 % kHelpers) % kHelpers;
-        rec = origin + a.nequil_w[ww] + (at + 1) * a.stride - 1;
+        walk.enter(origin, a.nequil_w[ww], a.stride, from, helper);
         base = a.off_w[ww] + (long long)r * a.tw[ww];
         wend = a.sequential ? origin + a.window_steps : end;
     };
@@ -296,12 +292,12 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
             }
         };
         for (;;) {
-            for (const long long seg = wend < stop ? wend : stop; rec < seg; rec += kHelpers * a.stride, at += kHelpers) {
-                const long long v = X[b][rec - n0 + 1][lane];
-                a.xout[base + at] = d ? (float)__longlong_as_double(v) : (float)v * (float)unit;
+            for (const long long seg = wend < stop ? wend : stop; walk.rec < seg; walk.next(a.stride)) {
+                const long long v = X[b][walk.rec - n0 + 1][lane];
+                a.xout[base + walk.at] = d ? (float)__longlong_as_double(v) : (float)v * (float)unit;
                 if (a.wout) {
-                    moves_to(rec + 1);
-                    a.wout[base + at] = d ? W : fixed_work();
+                    moves_to(walk.rec + 1);
+                    a.wout[base + walk.at] = d ? W : fixed_work();
                 }
             }
             if (!a.sequential || wend >= stop) break;
