@@ -633,6 +633,14 @@ pmf_status pmf_chain_forces(pmf_system *sys, int chain, const double *pos, doubl
  * PMF_EINVAL for helper outside 0..2, stride < 1 or negative counts. */
 pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t from, int n, int64_t *at, int64_t *step);
 
+/* The 1D integrator's fixed-point map on the host (no GPU needed): x'
+ * = x (1 + cB1 + cA x^2) + q in units of 2^(range_log2 - 62), n steps from X0 with
+ * terms q[n]; X[i] is the position after step i.  *outside is 1 if the range guard
+ * saw a position outside [-2^62, 2^62), from which on X means nothing.
+ * PMF_EINVAL if a coefficient times the range does not stay below 1. */
+pmf_status pmf_od1d_fixed_map(double cA, double cB1, int range_log2, int64_t X0, int n, const int64_t *q, int64_t *X,
+                              int *outside);
+
 /* Overlap coefficients ovl[i] = int min(p_i, p_{i+1}) dx, i < n - 1, of the
  * Gaussians N(mu_i, exp(log_var_i)) (host arrays), computed by the kernel
  * the adaptive protocol uses. */

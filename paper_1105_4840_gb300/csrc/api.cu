@@ -10,6 +10,7 @@
 
 #include "../../include/pmf.h"
 #include "common.cuh"
+#include "fixed62.h"
 #include "internal.h"
 
 using namespace pmf;
@@ -2129,6 +2130,24 @@ pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t fro
         at[i] = walk.at;
         step[i] = walk.rec;
     }
+    return PMF_OK;
+}
+
+pmf_status pmf_od1d_fixed_map(double cA, double cB1, int range_log2, int64_t X0, int n, const int64_t *q, int64_t *X,
+                              int *outside)
+{
+    if (n < 0 || (n > 0 && (!q || !X)) || !outside || std::abs(range_log2) > 30 || !(std::fabs(cB1) < 1.0) ||
+        !(std::fabs(std::ldexp(cA, 2 * range_log2)) < 1.0))
+        return fail(PMF_EINVAL, "pmf_od1d_fixed_map: bad argument");
+    const FixedStep f{limbs(std::llrint(std::ldexp(cA, 62 + 2 * range_log2))), std::llrint(std::ldexp(cB1, 62))};
+    unsigned guard = 0;
+    long long x = X0;
+    for (int i = 0; i < n; ++i) {
+        x = fixed_step(f, x, q[i]);
+        guard |= range_guard(x);
+        X[i] = x;
+    }
+    *outside = guard >> 31;
     return PMF_OK;
 }
 

@@ -24,6 +24,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "fixed62.h"
 #include "internal.h"
 
 namespace pmf {
@@ -84,48 +85,6 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
             q[(n - a.c0) * a.n_rep + rep] = a.fixed ? __double2ll_rn(qn) : __double_as_longlong(qn);
         }
     }
-}
-
-// A 62-bit fixed-point number as two 31-bit limbs, h 2^31 + l with
-// 0 <= l < 2^31.  a b 2^-62 of two such numbers (|a|, |b| < 2^62) is
-// a.h b.h + 2 (hi(a.h b.l) + hi(a.l b.h)), hi = the upper 32 bits of a 64-bit
-// product, within 5 units: the two cross products keep 30 bits each and the
-// product of the low limbs is dropped.
-struct Limbs {
-    int h, l;
-};
-__device__ __forceinline__ Limbs limbs(long long v) { return {(int)(v >> 31), (int)(v & 0x7fffffff)}; }
-__device__ __forceinline__ int mad_hi(int a, int b, int c)
-{
-    int d;
-    asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c)  // wraps
-{
-    long long d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ long long mul62_add(Limbs a, Limbs b, long long c)
-{
-    return mad_wide(mad_hi(a.l, b.h, __mulhi(a.h, b.l)), 2, mad_wide(a.h, b.h, c));
-}
-
-struct FixedStep {
-    Limbs ca;      // cA 4^b 2^62
-    long long cb;  // (cB - 1) 2^62
-};
-// One step, X' = X + Q + X w, w = (cB - 1) + cA x^2: three products, 19
-// integer instructions with the sums folded into the multiply-adds (64-bit
-// products by limbs cost twice that, most of it shifts and splits).  Sums wrap
-// where a trajectory leaves the range; the caller discards that tile.
-__device__ __forceinline__ long long fixed_step(const FixedStep &f, long long X, long long q)
-{
-    const Limbs x = limbs(X);
-    const Limbs y = limbs(mad_wide(__mulhi(x.h, x.l), 4, (long long)x.h * x.h));
-    const Limbs w = limbs(mul62_add(f.ca, y, f.cb));
-    return mul62_add(w, x, (long long)((unsigned long long)X + (unsigned long long)q));
 }
 
 // 32 simulations per CTA, steps [c0, c1): the parallel protocol (window rep /
@@ -193,22 +152,22 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         bool redo = dbl && lim > 0;
         if (!dbl) {
             X[b][0][lane] = Xi;
-            int guard = 0;  // sign bit: a position outside [-2^62, 2^62)
+            unsigned guard = 0;  // top bit: a position outside [-2^62, 2^62)
             if (__all_sync(__activemask(), lim == kTile)) {
 #pragma unroll 8
                 for (int s = 0; s < kTile; ++s) {
                     Xi = fixed_step(f, Xi, Q[b][s][lane]);
                     X[b][s + 1][lane] = Xi;
-                    guard |= (int)(Xi >> 32) + 0x40000000;
+                    guard |= range_guard(Xi);
                 }
             } else {
                 for (int s = 0; s < lim; ++s) {
                     Xi = fixed_step(f, Xi, Q[b][s][lane]);
                     X[b][s + 1][lane] = Xi;
-                    guard |= (int)(Xi >> 32) + 0x40000000;
+                    guard |= range_guard(Xi);
                 }
             }
-            if (guard < 0) {
+            if (guard >> 31) {
                 x = (double)X0 * unit;
                 dbl = redo = true;
             }

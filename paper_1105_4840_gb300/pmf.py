@@ -136,6 +136,7 @@ def _load():
     L.pmf_chain_schedule.argtypes = [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int), C.c_size_t,
                                      C.POINTER(C.c_size_t), C.POINTER(C.c_int)]
     L.pmf_od1d_records.argtypes = [C.c_int, C.c_int64, C.c_int, C.c_int64, C.c_int, _I64, _I64]
+    L.pmf_od1d_fixed_map.argtypes = [C.c_double, C.c_double, C.c_int, C.c_int64, C.c_int, _I64, _I64, C.POINTER(C.c_int)]
     L.pmf_run_reduce.argtypes = [P]
     L.pmf_run_set_queue_start.argtypes = [P, C.c_int64]
     L.pmf_run_set_batch_launch.argtypes = [P, C.c_int, C.c_int]
@@ -178,7 +179,7 @@ def _load():
                  "pmf_run_wait", "pmf_get_run_info", "pmf_x_samples", "pmf_work_samples",
                  "pmf_free_energy", "pmf_free_energy_from_samples", "pmf_final_state",
                  "pmf_run_partials", "pmf_free_energy_from_partials", "pmf_work_distributions", "pmf_philox",
-                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
+                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
                  "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc",
                  "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train",
@@ -708,6 +709,16 @@ def pmf_od1d_records(helper, n_equil, stride, start, n):
     _check(lib.pmf_od1d_records(helper, n_equil, stride, start, n, at.ctypes.data_as(_I64), step.ctypes.data_as(_I64)),
            "pmf_od1d_records")
     return at, step
+
+
+def pmf_od1d_fixed_map(cA, cB1, range_log2, X0, q):
+    """(positions after each step, left the range) of the 1D integrator's
+    fixed-point map on the host, in units of 2^(range_log2 - 62)."""
+    q = np.ascontiguousarray(q, dtype=np.int64)
+    X, out = np.zeros_like(q), C.c_int()
+    _check(lib.pmf_od1d_fixed_map(cA, cB1, range_log2, X0, q.size, q.ctypes.data_as(_I64), X.ctypes.data_as(_I64),
+                                  C.byref(out)), "pmf_od1d_fixed_map")
+    return X, bool(out.value)
 
 
 def pmf_fp32_peak(packed=True, ctas_per_sm=0, iters=1 << 16, reps=3):
