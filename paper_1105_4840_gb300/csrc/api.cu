@@ -2139,11 +2139,12 @@ pmf_status pmf_od1d_fixed_map(double cA, double cB1, int range_log2, int64_t X0,
     if (n < 0 || (n > 0 && (!q || !X)) || !outside || std::abs(range_log2) > 30 || !(std::fabs(cB1) < 1.0) ||
         !(std::fabs(std::ldexp(cA, 2 * range_log2)) < 1.0))
         return fail(PMF_EINVAL, "pmf_od1d_fixed_map: bad argument");
-    const FixedStep f{limbs(std::llrint(std::ldexp(cA, 62 + 2 * range_log2))), std::llrint(std::ldexp(cB1, 62))};
+    const FixedStep f = step_of(cA, cB1, range_log2);
+    const int off = q_offset256(cA, cB1);
     unsigned guard = 0;
     long long x = X0;
     for (int i = 0; i < n; ++i) {
-        x = fixed_step(f, x, q[i]);
+        x = fixed_step(f, x, q[i] + q_offset(off, i));
         guard |= range_guard(x);
         X[i] = x;
     }

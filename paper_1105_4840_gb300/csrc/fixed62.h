@@ -3,14 +3,17 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 
 namespace pmf {
 
 // A 62-bit fixed-point number as two 31-bit limbs, h 2^31 + l with
 // 0 <= l < 2^31.  a b 2^-62 of two such numbers (|a|, |b| < 2^62) is
 // a.h b.h + 2 (hi(a.h b.l) + hi(a.l b.h)), hi = the upper 32 bits of a 64-bit
-// product, within 5 units: the two cross products keep 30 bits each and the
-// product of the low limbs is dropped.
+// product: the two cross products keep 30 bits each and the product of the low
+// limbs is dropped.  Both round down: the result is 0 to 5 units low, 2 1/4 on
+// average (1 for each cross product, 1/4 for the low limbs), and what is added
+// to it makes up for that average (step_of, q_offset).
 struct Limbs {
     int h, l;
 };
@@ -50,8 +53,37 @@ __host__ __device__ __forceinline__ long long mul62_add(Limbs a, Limbs b, long l
 
 struct FixedStep {
     Limbs ca;      // cA 4^b 2^62
-    long long cb;  // (cB - 1) 2^62
+    long long cb;  // (cB - 1) 2^62, and the mean that w would be low by
 };
+__host__ __device__ __forceinline__ long long round_ll(double v)
+{
+#ifdef __CUDA_ARCH__
+    return __double2ll_rn(v);
+#else
+    return llrint(v);
+#endif
+}
+__host__ __device__ __forceinline__ FixedStep step_of(double cA, double cB1, int b)
+{
+    FixedStep f{limbs(round_ll(scalbn(cA, 62 + 2 * b))), round_ll(scalbn(cB1, 62))};
+    // w = ca y + cb is 2 1/4 low, and by ca times the 2 1/3 that y = x^2 is (its low limb is squared)
+    if (cA != 0.0) f.cb += (long long)(2.75f + 2.3333f * (float)f.ca.h * 0x1p-31f);
+    return f;
+}
+// The mean of a step's last product, x w, in 1/256 units.  With cA = 0 w is a
+// constant: a limb of zero loses nothing, and its low limb's mean is itself.
+__host__ __device__ __forceinline__ int q_offset256(double cA, double cB1)
+{
+    if (cA != 0.0) return 576;
+    const Limbs w = limbs(round_ll(scalbn(cB1, 62)));
+    return 256 * ((w.h != 0) + (w.l != 0)) + (w.l >> 24);
+}
+// Its share in step n's q_n: whole units, o256 over any 256 steps.
+__host__ __device__ __forceinline__ int q_offset(int o256, long long n)
+{
+    const int i = (int)(n & 255);
+    return ((o256 * (i + 1)) >> 8) - ((o256 * i) >> 8);
+}
 // One step, X' = X + Q + X w, w = (cB - 1) + cA x^2: three products, 19
 // integer instructions with the sums folded into the multiply-adds (64-bit
 // products by limbs cost twice that, most of it shifts and splits).  Sums wrap

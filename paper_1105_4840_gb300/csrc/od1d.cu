@@ -17,9 +17,12 @@
 // X = x 2^S with |x| < 2^b, S = 62 - b, and
 //   X' = X + Q + X w,  w = (cB - 1) + cA 4^b (X 2^-62)^2,
 // products of 62-bit numbers within a few units of 2^(b-62) (9e-19 for the
-// double well's b = 2), 1/128 of the FP64 rounding of a position near 1; the
-// results are no further from the exact map than FP64's.  A simulation that leaves |x| < 2^b redoes the
-// tile of steps it left in, and runs on, in FP64.
+// double well's b = 2), 1/128 of the FP64 rounding of a position near 1.  The
+// products round down; left alone that drift adds up to 2 1/4 units /
+// (k dt/gamma) where no well contracts the map faster (a = 0, k = 1, dt = 1e-3,
+// b = 4: 7.5e-15 against FP64's 1.2e-15), so its mean is added to the terms
+// that are there anyway, cB - 1 and q_n (the same case: 6e-17).  A simulation that leaves |x| < 2^b
+// redoes the tile of steps it left in, and runs on, in FP64.
 #include <algorithm>
 #include <cmath>
 
@@ -47,6 +50,7 @@ struct Od1dArgs {
     double smd_vdt;             //   trap advance per step after the equilibration
     long long *noise;           // [c1 - c0][n_rep] q_n of this launch's steps (fixed: q_n 2^S, else the double's bits)
     int fixed, range_log2;      // fixed point: on, and b
+    int q_off;                  // fixed point: mean of the last product's rounding (q_offset256)
     double cA, cB1;             // -4a dt/gamma, (4a - k) dt/gamma
     double amp, ck;             // sqrt(2 kT dt/gamma), k dt/gamma; fixed: times 2^S (set on the host: per thread
                                 // they took a sixth of the pre-pass's FP64 operations)
@@ -82,7 +86,7 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
         const long long n = n0 + l;
         if (n < a.c1) {
             const double qn = fma(a.amp, v[l], a.ck * trap_centre(a, rep, n));
-            q[(n - a.c0) * a.n_rep + rep] = a.fixed ? __double2ll_rn(qn) : __double_as_longlong(qn);
+            q[(n - a.c0) * a.n_rep + rep] = a.fixed ? __double2ll_rn(qn) + q_offset(a.q_off, n) : __double_as_longlong(qn);
         }
     }
 }
@@ -136,8 +140,7 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
     if (warp == 0 && live) {
         x = a.c0 == 0 ? (a.start ? a.start[rep] : a.x0) : a.state[2 * rep];
         if (a.fixed) {
-            f.ca = limbs(__double2ll_rn(scalbn(cA, 62 + 2 * a.range_log2)));
-            f.cb = __double2ll_rn(scalbn(cB1, 62));
+            f = step_of(cA, cB1, a.range_log2);
             if (fabs(x) < scalbn(1.0, a.range_log2)) {
                 Xi = __double2ll_rn(x * scale);
                 dbl = false;
@@ -177,7 +180,7 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
 #pragma unroll 4
             for (int s = 0; s < lim; ++s) {
                 const long long qb = Q[b][s][lane];
-                x = fma(x, fma(cA, x * x, cB), a.fixed ? (double)qb * unit : __longlong_as_double(qb));
+                x = fma(x, fma(cA, x * x, cB), a.fixed ? (double)(qb - q_offset(a.q_off, n0 + s)) * unit : __longlong_as_double(qb));
                 X[b][s + 1][lane] = __double_as_longlong(x);
             }
         }
@@ -340,6 +343,7 @@ cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cuda
     }
     a.cA = -4.0 * m.a * dtg;
     a.cB1 = (4.0 * m.a - L.k) * dtg;
+    a.q_off = a.fixed ? q_offset256(a.cA, a.cB1) : 0;
     const double scale = a.fixed ? std::ldexp(1.0, 62 - a.range_log2) : 1.0;
     a.amp = std::sqrt(2.0 * L.kT * dtg) * scale;
     a.ck = L.k * dtg * scale;

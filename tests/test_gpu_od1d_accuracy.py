@@ -1,0 +1,34 @@
+"""End positions of the 1D integrator against its map in exact arithmetic."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from paper_1105_4840_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pmf():
+    from paper_1105_4840_gb300 import pmf as m
+    return m
+
+
+@pytest.mark.parametrize("lam,b", [(8.0, 4), (-6.3, 3), (0.7, 0)])
+def test_trap_without_wells(pmf, lam, b):
+    """A pure trap (a = 0, k dt = 1e-3) without noise remembers 1000 steps, so a
+    rounding that always goes one way adds up to 1000 of its means (the
+    products' 2 1/4 units of 2^(b-62) would give 7.8e-15 at b = 4).  Rounding to either side
+    leaves 1.2 units x sqrt(1000 / 2), five times that is 134 units, and 4 units for
+    the offset's own 1/256; the end position is then rounded to a double."""
+    run = inputs.RunSettings(k=1.0, kT=1e-40, dt=1e-3, gamma=1.0, n_steps=20000, n_equil=0, stride=100, replicas=2, seed=3)
+    sysh = pmf.pmf_create_system_1d(0.0, 0.25)
+    rr = pmf.pmf_run_windows(sysh, np.array([lam]), pmf.make_params(run))
+    c, one = Fraction(-1e-3), 2**180  # the coefficient as the kernel has it; positions in units of 2^-180
+    q = int(Fraction(1e-3 * lam) * one)
+    x = one // 4
+    for _ in range(run.n_steps):
+        x += (x * c.numerator) // c.denominator + q
+    for got in rr.final_state()[0]:
+        assert abs(Fraction(float(got)) - Fraction(x, one)) <= 138 * Fraction(2) ** (b - 62) + Fraction(np.spacing(abs(got)) / 2)
