@@ -633,6 +633,12 @@ pmf_status pmf_chain_forces(pmf_system *sys, int chain, const double *pos, doubl
  * PMF_EINVAL for helper outside 0..2, stride < 1 or negative counts. */
 pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t from, int n, int64_t *at, int64_t *step);
 
+/* The range b, |x| < 2^b, of the fixed point that the 1D integrator computes a
+ * simulation in whose trap centres lie between near and far from 0, or -1000
+ * where it computes in FP64 (host, no GPU needed). */
+pmf_status pmf_od1d_range(double a, double x0, double k, double kT, double dt, double gamma, double far, double near,
+                          int *range_log2);
+
 /* The 1D integrator's fixed-point map on the host (no GPU needed): x'
  * = x (1 + cB1 + cA x^2) + q in units of 2^(range_log2 - 62), n steps from X0 with
  * terms q[n]; X[i] is the position after step i.  *outside is 1 if the range guard

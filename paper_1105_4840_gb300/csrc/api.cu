@@ -447,9 +447,12 @@ static RunLaunch item_launch(const pmf_run *run, const RunItem &ri)
     L.abort = run->d_abort;
     L.wout = run->d_w;       // set for pulled runs only
     L.smd_vdt = run->smd_vdt;
-    for (int i = ri.w0; i < ri.w0 + ri.nw; ++i)
-        L.lambda_max = std::max({L.lambda_max, std::fabs(run->lambda[i]),
-                                 std::fabs(run->lambda[i] + run->smd_vdt * (double)run->nsteps[i])});
+    L.lambda_min = INFINITY;
+    for (int i = ri.w0; i < ri.w0 + ri.nw; ++i) {  // from centre u to centre v
+        const double u = run->lambda[i], v = u + run->smd_vdt * (double)run->nsteps[i];
+        L.lambda_max = std::max({L.lambda_max, std::fabs(u), std::fabs(v)});
+        L.lambda_min = std::min(L.lambda_min, (u < 0) != (v < 0) ? 0.0 : std::min(std::fabs(u), std::fabs(v)));
+    }
     // 1D runs: this item's block of the noise buffer
     L.noise = run->d_noise ? run->d_noise + (size_t)run->noise_steps * ri.w0 * run->replicas : nullptr;
     L.noise_steps = run->noise_steps;
@@ -2130,6 +2133,18 @@ pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t fro
         at[i] = walk.at;
         step[i] = walk.rec;
     }
+    return PMF_OK;
+}
+
+pmf_status pmf_od1d_range(double a, double x0, double k, double kT, double dt, double gamma, double far, double near,
+                          int *range_log2)
+{
+    if (!(k > 0) || !(kT > 0) || !(dt > 0) || !(gamma > 0) || !(far >= near) || !(near >= 0) || !range_log2)
+        return fail(PMF_EINVAL, "pmf_od1d_range: bad argument");
+    Od1dParams m;
+    m.a = a;
+    m.x0 = x0;
+    *range_log2 = fixed_range(od1d_range_rule(m, k, kT, dt, gamma), far, near);
     return PMF_OK;
 }
 

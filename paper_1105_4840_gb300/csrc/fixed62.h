@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <string.h>
 
 namespace pmf {
 
@@ -100,6 +101,40 @@ __host__ __device__ __forceinline__ long long fixed_step(const FixedStep &f, lon
 __host__ __device__ __forceinline__ unsigned range_guard(long long X)
 {
     return (unsigned)((unsigned long long)X >> 32) + 0x40000000u;
+}
+
+// Which b (|x| < 2^b) a simulation's fixed point takes.  It depends on the
+// model, the run's parameters and the simulation's own trap centres alone, so a
+// window's trajectory has the same bits in every launch that holds it.
+constexpr int kNoRange = -1000;  // FP64 instead
+struct RangeRule {
+    double hold = 0, pad = 0;    // 2^b > max(|trap centre|, hold) + pad: start and wells, six widths of the trap
+    double width = 0, well = 0;  // |x| is of the order of max(width, min(|trap centre|, well))
+    unsigned long long fits = 0; // bit b + 30: no step from inside the range wraps a 64-bit sum
+};
+__host__ __device__ __forceinline__ long long double_bits(double v)
+{
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(v);
+#else
+    long long b;
+    memcpy(&b, &v, sizeof(b));
+    return b;
+#endif
+}
+// e with v < 2^e (v >= 0), and max and min of non-negative numbers, on the integer pipe.
+__host__ __device__ __forceinline__ int exponent_above(double v) { return (int)(double_bits(v) >> 52) - 1022; }
+__host__ __device__ __forceinline__ double max_bits(double a, double b) { return double_bits(a) > double_bits(b) ? a : b; }
+__host__ __device__ __forceinline__ double min_bits(double a, double b) { return double_bits(a) < double_bits(b) ? a : b; }
+// far, near: largest and smallest |trap centre| of the simulation.  A step of the
+// fixed point is off by 1.2 units of 2^(b-62) rms, one of FP64 by |x| 2^-53.7, so FP64 is
+// as close where 2^b = 256 |x| (measured without wells, 2^b / width 128, 256,
+// 512: 0.48, 0.90, 1.8 times FP64's error); the line is at half of that.
+__host__ __device__ __forceinline__ int fixed_range(const RangeRule &r, double far, double near)
+{
+    const int b = exponent_above(max_bits(far, r.hold) + r.pad);
+    const double size = max_bits(r.width, min_bits(near, r.well));
+    return b >= -30 && b <= 30 && ((r.fits >> (b + 30)) & 1) && b <= exponent_above(size) + 6 ? b : kNoRange;
 }
 
 }  // namespace pmf

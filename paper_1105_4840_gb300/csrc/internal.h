@@ -69,7 +69,7 @@ struct RunLaunch {
     // constant-velocity pulling (one window): the trap advances smd_vdt per
     // step after the equilibration; accumulated work recorded into wout
     double smd_vdt = 0;
-    double lambda_max = 0;  // 1D model: largest |trap centre| of the launch
+    double lambda_max = 0, lambda_min = 0;  // 1D model: largest and smallest |trap centre| of the launch
     double *wout = nullptr;
     // 1D model: buffer for the per-step noise-and-trap terms q_n of noise_steps
     // steps of every simulation
@@ -149,6 +149,8 @@ struct Od1dParams {
 // steps; the state holds x and the pulling work per simulation (2 doubles).
 cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cudaStream_t st);
 long long od1d_noise_steps(int n_rep);
+struct RangeRule;
+RangeRule od1d_range_rule(const Od1dParams &m, double k, double kT, double dt, double gamma);
 // Records of one window of a 1D simulation that one helper warp of kOd1dHelpers
 // takes (record number `at`: helper at mod kOd1dHelpers).  rec: the step whose end
 // it is taken at; 64 bits throughout: strides go up to 2^31 - 1, step counts

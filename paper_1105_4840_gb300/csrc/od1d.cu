@@ -12,8 +12,8 @@
 //
 // Arithmetic of the chain.  This GPU's FP64 unit takes 64 cycles per operation
 // of a warp, dependent or not, so the three FP64 operations of a step cost 192
-// cycles.  Where the launch's parameters bound the motion, the chain runs in
-// 62-bit fixed point on the integer pipe instead (IMAD.WIDE: 5 cycles):
+// cycles.  Where a simulation's parameters bound its motion (fixed_range), its
+// chain runs in 62-bit fixed point on the integer pipe instead (IMAD.WIDE: 5 cycles):
 // X = x 2^S with |x| < 2^b, S = 62 - b, and
 //   X' = X + Q + X w,  w = (cB - 1) + cA 4^b (X 2^-62)^2,
 // products of 62-bit numbers within a few units of 2^(b-62) (9e-19 for the
@@ -48,13 +48,24 @@ struct Od1dArgs {
     long long window_steps;
     double *wout;               // constant-velocity pulling: work at the records
     double smd_vdt;             //   trap advance per step after the equilibration
-    long long *noise;           // [c1 - c0][n_rep] q_n of this launch's steps (fixed: q_n 2^S, else the double's bits)
-    int fixed, range_log2;      // fixed point: on, and b
-    int q_off;                  // fixed point: mean of the last product's rounding (q_offset256)
+    long long *noise;           // [c1 - c0][n_rep] q_n of this launch's steps (fixed point: q_n 2^S, else the double's bits)
+    RangeRule rule;             // fixed point: range of a window,
+    int range;                  //   or of the whole run (sequential, pulled)
+    int q_off;                  //   mean of the last product's rounding (q_offset256)
     double cA, cB1;             // -4a dt/gamma, (4a - k) dt/gamma
-    double amp, ck;             // sqrt(2 kT dt/gamma), k dt/gamma; fixed: times 2^S (set on the host: per thread
+    double amp, ck;             // sqrt(2 kT dt/gamma), k dt/gamma (set on the host: per thread
                                 // they took a sixth of the pre-pass's FP64 operations)
 };
+
+// b of simulation rep, or kNoRange.
+__device__ __forceinline__ int range_of(const Od1dArgs &a, int rep)
+{
+    if (a.sequential || a.wout) return a.range;
+    const double l = fabs(a.lambda[rep / a.replicas]);
+    return fixed_range(a.rule, l, l);
+}
+// v 2^s for a normal v (and result), or zero left alone, without the FP64 unit
+__device__ __forceinline__ double scaled(double v, int s) { return __hiloint2double(__double2hiint(v) + (s << 20), __double2loint(v)); }
 
 // Trap centre during step n of simulation rep: its window's lambda (the
 // window of step n in the sequential protocol), or, when pulled, lambda_1
@@ -81,12 +92,14 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
     const Normal4<double> z =
         philox_normals<double>(a.seed, 0u, a.uid_base + (uint32_t)rep, (uint32_t)(n0 >> 2), kTagOStep);
     const double v[4] = {z.n0, z.n1, z.n2, z.n3};
+    const int b = range_of(a, rep), S = b == kNoRange ? 0 : 62 - b;
+    const double amp = scaled(a.amp, S), ck = scaled(a.ck, S);
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
         const long long n = n0 + l;
         if (n < a.c1) {
-            const double qn = fma(a.amp, v[l], a.ck * trap_centre(a, rep, n));
-            q[(n - a.c0) * a.n_rep + rep] = a.fixed ? __double2ll_rn(qn) + q_offset(a.q_off, n) : __double_as_longlong(qn);
+            const double qn = fma(amp, v[l], ck * trap_centre(a, rep, n));
+            q[(n - a.c0) * a.n_rep + rep] = b != kNoRange ? __double2ll_rn(qn) + q_offset(a.q_off, n) : __double_as_longlong(qn);
         }
     }
 }
@@ -108,91 +121,115 @@ constexpr int kTile = 40;  // 41.5 KB of shared memory a CTA; 32 steps: 2.17 aga
 static_assert(kTile % 8 == 0, "unrolled by 8");
 constexpr int kOd1dThreads = 128;
 
-__global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
+// Two tiles' buffers in shared memory.
+struct Od1dTiles {
+    long long (&Q)[2][kTile][32];      // q_n
+    long long (&X)[2][kTile + 1][32];  // positions before the tile's first step and after each
+    unsigned (&dbl_mask)[2];           // lanes whose tile is in FP64 (bits of doubles)
+};
+// What both roles know of a lane's simulation.
+struct Od1dSim {
+    int lane, rep, w, range;  // w: its window (0 in the sequential protocol)
+    bool live, fixed;
+    long long end, tiles;     // its last step (its window's step count), the launch's tiles
+    double scale, unit;       // 2^S and 2^-S
+};
+__device__ __forceinline__ void tile_barrier() { asm volatile("bar.sync 0, %0;" ::"n"(kOd1dThreads) : "memory"); }
+// Rows row, row + STEP, ... of tile i: all loads, then all stores.  A load and its
+// store at a time are 14 latencies a helper, longer than the integrating
+// warp's 40 steps (21 x 8 x 2e4 steps: 2350 us, now 1712).
+template <int STEP>
+__device__ __forceinline__ void load_tile(const Od1dArgs &a, const Od1dTiles &sh, const Od1dSim &m, long long i, int row)
 {
-    __shared__ long long Q[2][kTile][32];      // q_n
-    __shared__ long long X[2][kTile + 1][32];  // positions before the tile's first step and after each
-    __shared__ unsigned dbl_mask[2];           // lanes whose tile is in FP64 (bits of doubles)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rep = blockIdx.x * 32 + lane;
-    const bool live = rep < a.n_rep;
-    const int r = a.sequential ? rep : rep % a.replicas;
-    const int w = a.sequential || !live ? 0 : rep / a.replicas;
-    // this simulation's last step (its window's step count)
-    long long end = a.c1;
-    if (!a.sequential && live) end = end < a.nsteps_w[w] ? end : a.nsteps_w[w];
-    if (!live || end < a.c0) end = a.c0;
-    const double scale = scalbn(1.0, 62 - a.range_log2), unit = scalbn(1.0, a.range_log2 - 62);
-    const double cA = a.cA, cB1 = a.cB1, cB = 1.0 + cB1;
-    const long long tiles = (a.c1 - a.c0 + kTile - 1) / kTile;
+    constexpr int kRows = (kTile + STEP - 1) / STEP;
+    const long long n0 = i * kTile, left = a.c1 - a.c0 - n0;
+    const int rows = !m.live ? 0 : (left < kTile ? (int)left : kTile);
+    const long long *q = a.noise + (n0 + row) * a.n_rep + m.rep;
+    long long v[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+        if (row + u * STEP < rows) v[u] = q[(long long)u * STEP * a.n_rep];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+        if (row + u * STEP < rows) sh.Q[i & 1][row + u * STEP][m.lane] = v[u];
+}
 
-    auto load_tile = [&](long long i, int row, int step) {
-        const long long n0 = i * kTile;
-        for (int s = row; s < kTile; s += step)
-            if (live && n0 + s < a.c1 - a.c0) Q[i & 1][s][lane] = a.noise[(n0 + s) * a.n_rep + rep];
-    };
-
-    // warp 0: the position, in fixed point or (dbl) FP64
+// Warp 0: the position, in fixed point or (dbl) FP64.
+__device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTiles &sh, const Od1dSim &m)
+{
+    const int lane = m.lane;
+    const double cA = a.cA, cB = 1.0 + a.cB1;
     FixedStep f{};
     long long Xi = 0;
     double x = 0.0;
     bool dbl = true;
-    if (warp == 0 && live) {
-        x = a.c0 == 0 ? (a.start ? a.start[rep] : a.x0) : a.state[2 * rep];
-        if (a.fixed) {
-            f = step_of(cA, cB1, a.range_log2);
-            if (fabs(x) < scalbn(1.0, a.range_log2)) {
-                Xi = __double2ll_rn(x * scale);
+    if (m.live) {
+        x = a.c0 == 0 ? (a.start ? a.start[m.rep] : a.x0) : a.state[2 * m.rep];
+        if (m.fixed) {
+            f = step_of(cA, a.cB1, m.range);
+            if (fabs(x) < scaled(1.0, m.range)) {
+                Xi = __double2ll_rn(x * m.scale);
                 dbl = false;
             }
         }
     }
-    auto integrate = [&](long long i) {
+    for (long long i = 0; i < m.tiles; ++i) {
         const long long n0 = a.c0 + i * kTile;
         const int b = (int)(i & 1);
-        const int lim = end <= n0 ? 0 : (end - n0 < kTile ? (int)(end - n0) : kTile);
+        const int lim = m.end <= n0 ? 0 : (m.end - n0 < kTile ? (int)(m.end - n0) : kTile);
         const long long X0 = Xi;
         bool redo = dbl && lim > 0;
         if (!dbl) {
-            X[b][0][lane] = Xi;
+            sh.X[b][0][lane] = Xi;
             unsigned guard = 0;  // top bit: a position outside [-2^62, 2^62)
             if (__all_sync(__activemask(), lim == kTile)) {
 #pragma unroll 8
                 for (int s = 0; s < kTile; ++s) {
-                    Xi = fixed_step(f, Xi, Q[b][s][lane]);
-                    X[b][s + 1][lane] = Xi;
+                    Xi = fixed_step(f, Xi, sh.Q[b][s][lane]);
+                    sh.X[b][s + 1][lane] = Xi;
                     guard |= range_guard(Xi);
                 }
             } else {
                 for (int s = 0; s < lim; ++s) {
-                    Xi = fixed_step(f, Xi, Q[b][s][lane]);
-                    X[b][s + 1][lane] = Xi;
+                    Xi = fixed_step(f, Xi, sh.Q[b][s][lane]);
+                    sh.X[b][s + 1][lane] = Xi;
                     guard |= range_guard(Xi);
                 }
             }
-            if (guard >> 31) {
-                x = (double)X0 * unit;
-                dbl = redo = true;
-            }
+            redo = guard >> 31;
         }
         if (redo) {
-            X[b][0][lane] = __double_as_longlong(x);
+            if (!dbl) x = (double)X0 * m.unit;
+            dbl = true;
+            sh.X[b][0][lane] = __double_as_longlong(x);
 #pragma unroll 4
             for (int s = 0; s < lim; ++s) {
-                const long long qb = Q[b][s][lane];
-                x = fma(x, fma(cA, x * x, cB), a.fixed ? (double)(qb - q_offset(a.q_off, n0 + s)) * unit : __longlong_as_double(qb));
-                X[b][s + 1][lane] = __double_as_longlong(x);
+                const long long qb = sh.Q[b][s][lane];
+                const double q = m.fixed ? (double)(qb - q_offset(a.q_off, n0 + s)) * m.unit : __longlong_as_double(qb);
+                x = fma(x, fma(cA, x * x, cB), q);
+                sh.X[b][s + 1][lane] = __double_as_longlong(x);
             }
         }
         __syncwarp();
         const unsigned mask = __ballot_sync(0xffffffffu, dbl);
-        if (lane == 0) dbl_mask[b] = mask;
-    };
+        if (lane == 0) sh.dbl_mask[b] = mask;
+        tile_barrier();
+    }
+    tile_barrier();  // (the last tile's records)
+    if (!m.live || m.end <= a.c0) return;
+    if (!dbl) x = (double)Xi * m.unit;
+    if (!isfinite(x)) atomicOr(a.err, kErrNonFinite);
+    a.state[2 * m.rep] = x;
+    if (!a.wout) a.state[2 * m.rep + 1] = 0.0;
+}
 
-    // warps 1 - 3: the records of a finished tile; no division in the loop
-    const int helper = warp - 1;
-    static_assert(kOd1dHelpers == kOd1dThreads / 32 - 1, "every warp but the first records");
-    int ww = w;
+// Warps 1 - 3: the next tile's q_n, and the records of the finished one; no
+// division in the loop.
+__device__ __forceinline__ void record_tiles(const Od1dArgs &a, const Od1dTiles &sh, const Od1dSim &m, int helper)
+{
+    const int lane = m.lane, r = a.sequential ? m.rep : m.rep % a.replicas;
+    const float unit_f = __int_as_float(m.fixed ? (m.range - 62 + 127) << 23 : 0x3f800000);
+    int ww = m.w;
     RecordWalk walk;
     long long base = 0, wend = 0;
     auto enter_window = [&](int window, long long from) {
@@ -200,7 +237,7 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         const long long origin = a.sequential ? (long long)ww * a.window_steps : 0;
         walk.enter(origin, a.nequil_w[ww], a.stride, from, helper);
         base = a.off_w[ww] + (long long)r * a.tw[ww];
-        wend = a.sequential ? origin + a.window_steps : end;
+        wend = a.sequential ? origin + a.window_steps : m.end;
     };
     // pulling work: W after the trap's first moves0 moves, and since then the
     // sum of X - lambda_1 in two 32-bit halves (every helper keeps it, each
@@ -209,26 +246,26 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
     long long acc_h = 0, moves0 = 0, moves = 0;
     unsigned long long acc_l = 0;
     const double lam1 = a.lambda[0], kv = a.k * a.smd_vdt;
-    const long long L1 = a.fixed ? __double2ll_rn(lam1 * scale) : 0;
-    if (warp > 0 && live) {
-        enter_window(a.sequential ? (int)(a.c0 / a.window_steps) : w, a.c0);
+    const long long L1 = m.fixed ? __double2ll_rn(lam1 * m.scale) : 0;
+    if (m.live) {
+        enter_window(a.sequential ? (int)(a.c0 / a.window_steps) : m.w, a.c0);
         if (a.wout) {
-            W = a.c0 == 0 ? 0.0 : a.state[2 * rep + 1];
+            W = a.c0 == 0 ? 0.0 : a.state[2 * m.rep + 1];
             moves = a.c0 - 1 - a.nequil_w[0];
             moves0 = moves = moves > 0 ? moves : 0;
         }
     }
     // sum over the moves m of k vdt (lambda_1 + vdt (m - 1/2) - x)
     auto fixed_work = [&] {
-        const double m = (double)moves, m0 = (double)moves0;
-        const double sum = ((double)acc_h * 4294967296.0 + (double)acc_l) * unit;
-        return W + kv * (0.5 * a.smd_vdt * (m * m - m0 * m0) - sum);
+        const double mm = (double)moves, m0 = (double)moves0;
+        const double sum = ((double)acc_h * 4294967296.0 + (double)acc_l) * m.unit;
+        return W + kv * (0.5 * a.smd_vdt * (mm * mm - m0 * m0) - sum);
     };
     auto records = [&](long long i) {
-        if (!live) return;  // (such a lane has no window to record in)
+        if (!m.live) return;  // (such a lane has no window to record in)
         const int b = (int)(i & 1);
-        const bool d = (dbl_mask[b] >> lane) & 1;
-        const long long n0 = a.c0 + i * kTile, stop = end < n0 + kTile ? end : n0 + kTile;
+        const bool d = (sh.dbl_mask[b] >> lane) & 1;
+        const long long n0 = a.c0 + i * kTile, stop = m.end < n0 + kTile ? m.end : n0 + kTile;
         long long n = n0;  // positions before this step are in the work
         if (a.wout && d && moves != moves0) {  // FP64 from here on
             W = fixed_work();
@@ -240,7 +277,7 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         auto moves_to = [&](long long to) {                      // the trap's moves before steps [n, to)
             if (n < move1) n = move1;
             for (; n < to; ++n) {
-                const long long v = X[b][n - n0][lane];
+                const long long v = sh.X[b][n - n0][lane];
                 moves = n - move1 + 1;
                 if (d) {
                     const double lo = lam1 + a.smd_vdt * (double)(moves - 1), hi = lam1 + a.smd_vdt * (double)moves;
@@ -255,8 +292,8 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         };
         for (;;) {
             for (const long long seg = wend < stop ? wend : stop; walk.rec < seg; walk.next(a.stride)) {
-                const long long v = X[b][walk.rec - n0 + 1][lane];
-                a.xout[base + walk.at] = d ? (float)__longlong_as_double(v) : (float)v * (float)unit;
+                const long long v = sh.X[b][walk.rec - n0 + 1][lane];
+                a.xout[base + walk.at] = d ? (float)__longlong_as_double(v) : (float)v * unit_f;
                 if (a.wout) {
                     moves_to(walk.rec + 1);
                     a.wout[base + walk.at] = d ? W : fixed_work();
@@ -267,27 +304,38 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
         }
         if (a.wout) moves_to(stop);
     };
+    for (long long i = 0; i <= m.tiles; ++i) {
+        if (i + 1 < m.tiles) load_tile<kOd1dHelpers>(a, sh, m, i + 1, helper);
+        if (i > 0) records(i - 1);
+        tile_barrier();
+    }
+    if (helper == 0 && a.wout && m.live && m.end > a.c0) a.state[2 * m.rep + 1] = moves != moves0 ? fixed_work() : W;
+}
 
-    load_tile(0, warp, kOd1dThreads / 32);
-    __syncthreads();
-    for (long long i = 0; i <= tiles; ++i) {
-        if (warp == 0) {
-            if (i < tiles) integrate(i);
-        } else {
-            if (i + 1 < tiles) load_tile(i + 1, warp - 1, kOd1dThreads / 32 - 1);
-            if (i > 0) records(i - 1);
-        }
-        __syncthreads();
-    }
-    if (!live || end <= a.c0) return;
-    if (warp == 0) {
-        if (!dbl) x = (double)Xi * unit;
-        if (!isfinite(x)) atomicOr(a.err, kErrNonFinite);
-        a.state[2 * rep] = x;
-        if (!a.wout) a.state[2 * rep + 1] = 0.0;
-    } else if (warp == 1 && a.wout) {
-        a.state[2 * rep + 1] = moves != moves0 ? fixed_work() : W;
-    }
+__global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
+{
+    static_assert(kOd1dHelpers == kOd1dThreads / 32 - 1, "every warp but the first records");
+    __shared__ long long Q[2][kTile][32], X[2][kTile + 1][32];
+    __shared__ unsigned dbl_mask[2];
+    const Od1dTiles sh{Q, X, dbl_mask};
+    const int warp = threadIdx.x >> 5;
+    Od1dSim m;
+    m.lane = threadIdx.x & 31;
+    m.rep = blockIdx.x * 32 + m.lane;
+    m.live = m.rep < a.n_rep;
+    m.w = a.sequential || !m.live ? 0 : m.rep / a.replicas;
+    m.end = a.c1;
+    if (!a.sequential && m.live) m.end = m.end < a.nsteps_w[m.w] ? m.end : a.nsteps_w[m.w];
+    if (!m.live || m.end < a.c0) m.end = a.c0;
+    m.tiles = (a.c1 - a.c0 + kTile - 1) / kTile;
+    m.range = m.live ? range_of(a, m.rep) : kNoRange;
+    m.fixed = m.range != kNoRange;
+    m.scale = scaled(1.0, m.fixed ? 62 - m.range : 0);
+    m.unit = scaled(1.0, m.fixed ? m.range - 62 : 0);
+    load_tile<kOd1dThreads / 32>(a, sh, m, 0, warp);
+    tile_barrier();
+    if (warp == 0) integrate_tiles(a, sh, m);
+    else record_tiles(a, sh, m, warp - 1);
 }
 
 long long od1d_noise_steps(int n_rep)
@@ -296,6 +344,26 @@ long long od1d_noise_steps(int n_rep)
     long long c = (1LL << 23) / (n_rep > 0 ? n_rep : 1);
     c = c < 64 ? 64 : (c > 8192 ? 8192 : c);
     return c & ~3LL;
+}
+
+// The range holds the trap, the start, the wells and six widths of the trap, and
+// one step from inside cannot wrap a 64-bit sum (which also bounds every
+// coefficient): FP64 otherwise, for instance for time steps near the scheme's
+// stability limit.  Box-Muller's normals stay below sqrt(66 ln 2) < 6.8.
+RangeRule od1d_range_rule(const Od1dParams &m, double k, double kT, double dt, double gamma)
+{
+    RangeRule r;
+    const double dtg = dt / gamma, amp = std::sqrt(2.0 * kT * dtg), ck = k * dtg;
+    r.hold = std::max(std::fabs(m.x0), m.a != 0.0 ? 1.0 : 0.0);
+    r.pad = 6.0 * std::sqrt(kT / k);
+    r.width = std::sqrt(kT / (k + 4.0 * std::fabs(m.a)));
+    // between the trap and the wells, which an inverted potential has not
+    r.well = m.a == 0.0 ? INFINITY : (m.a > 0.0 ? 1.0 : 0.0);
+    const double cA = std::fabs(4.0 * m.a * dtg), cB1 = std::fabs((4.0 * m.a - k) * dtg);
+    if (!std::isnormal(amp) || !std::isnormal(ck)) return r;
+    for (int b = -30; b <= 30; ++b)
+        if (cB1 + std::ldexp(cA, 2 * b) + 6.8 * std::ldexp(amp, -b) + ck < 0.99) r.fits |= 1ull << (b + 30);
+    return r;
 }
 
 cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cudaStream_t st)
@@ -325,28 +393,14 @@ cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cuda
     a.wout = L.wout;
     a.smd_vdt = L.smd_vdt;
     a.noise = reinterpret_cast<long long *>(L.noise);
-    // Fixed point where |x| < 2^b holds the traps, the start, the wells and six
-    // widths of the trap, and where one step from inside cannot wrap a 64-bit
-    // sum (which also bounds every coefficient): FP64 otherwise, for instance
-    // for time steps near the scheme's stability limit.  Box-Muller's normals
-    // stay below sqrt(66 ln 2) < 6.8.
-    const double dtg = L.dt / L.gamma, reach = std::max({L.lambda_max, std::fabs(m.x0), m.a != 0.0 ? 1.0 : 0.0}) + 6.0 * std::sqrt(L.kT / L.k);
-    const double cA = std::fabs(4.0 * m.a * dtg), cB1 = std::fabs((4.0 * m.a - L.k) * dtg);
-    const double qmax = 6.8 * std::sqrt(2.0 * L.kT * dtg) + L.k * dtg * L.lambda_max;
-    if (std::isfinite(reach) && reach > 0 && std::isfinite(cA) && std::isfinite(cB1) && std::isfinite(qmax)) {
-        int b = 0;
-        std::frexp(reach, &b);  // reach <= 2^b
-        if (b >= -30 && b <= 30 && cB1 + std::ldexp(cA, 2 * b) + std::ldexp(qmax, -b) < 0.99) {
-            a.fixed = 1;
-            a.range_log2 = b;
-        }
-    }
+    const double dtg = L.dt / L.gamma;
     a.cA = -4.0 * m.a * dtg;
     a.cB1 = (4.0 * m.a - L.k) * dtg;
-    a.q_off = a.fixed ? q_offset256(a.cA, a.cB1) : 0;
-    const double scale = a.fixed ? std::ldexp(1.0, 62 - a.range_log2) : 1.0;
-    a.amp = std::sqrt(2.0 * L.kT * dtg) * scale;
-    a.ck = L.k * dtg * scale;
+    a.amp = std::sqrt(2.0 * L.kT * dtg);
+    a.ck = L.k * dtg;
+    a.rule = od1d_range_rule(m, L.k, L.kT, L.dt, L.gamma);
+    a.range = fixed_range(a.rule, L.lambda_max, L.lambda_min);
+    a.q_off = a.rule.fits ? q_offset256(a.cA, a.cB1) : 0;
     for (long long c0 = L.step_begin; c0 < L.step_end; c0 += L.noise_steps) {
         const long long c1 = c0 + L.noise_steps < L.step_end ? c0 + L.noise_steps : L.step_end;
         const long long cells = ((c1 - c0 + 3) >> 2) * n_rep;

@@ -136,6 +136,7 @@ def _load():
     L.pmf_chain_schedule.argtypes = [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int), C.c_size_t,
                                      C.POINTER(C.c_size_t), C.POINTER(C.c_int)]
     L.pmf_od1d_records.argtypes = [C.c_int, C.c_int64, C.c_int, C.c_int64, C.c_int, _I64, _I64]
+    L.pmf_od1d_range.argtypes = [C.c_double] * 8 + [C.POINTER(C.c_int)]
     L.pmf_od1d_fixed_map.argtypes = [C.c_double, C.c_double, C.c_int, C.c_int64, C.c_int, _I64, _I64, C.POINTER(C.c_int)]
     L.pmf_run_reduce.argtypes = [P]
     L.pmf_run_set_queue_start.argtypes = [P, C.c_int64]
@@ -179,7 +180,7 @@ def _load():
                  "pmf_run_wait", "pmf_get_run_info", "pmf_x_samples", "pmf_work_samples",
                  "pmf_free_energy", "pmf_free_energy_from_samples", "pmf_final_state",
                  "pmf_run_partials", "pmf_free_energy_from_partials", "pmf_work_distributions", "pmf_philox",
-                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
+                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
                  "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc",
                  "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train",
@@ -709,6 +710,14 @@ def pmf_od1d_records(helper, n_equil, stride, start, n):
     _check(lib.pmf_od1d_records(helper, n_equil, stride, start, n, at.ctypes.data_as(_I64), step.ctypes.data_as(_I64)),
            "pmf_od1d_records")
     return at, step
+
+
+def pmf_od1d_range(a, x0, k, kT, dt, gamma, far, near):
+    """Range b, |x| < 2^b, of a 1D simulation's fixed point, or None where it is
+    computed in FP64."""
+    b = C.c_int()
+    _check(lib.pmf_od1d_range(a, x0, k, kT, dt, gamma, far, near, C.byref(b)), "pmf_od1d_range")
+    return b.value if b.value != -1000 else None
 
 
 def pmf_od1d_fixed_map(cA, cB1, range_log2, X0, q):

@@ -1,4 +1,5 @@
-"""End positions of the 1D integrator against its map in exact arithmetic."""
+"""End positions of the 1D integrator against its map in exact arithmetic, and
+their bits in launches of different company."""
 from fractions import Fraction
 
 import numpy as np
@@ -32,3 +33,20 @@ def test_trap_without_wells(pmf, lam, b):
         x += (x * c.numerator) // c.denominator + q
     for got in rr.final_state()[0]:
         assert abs(Fraction(float(got)) - Fraction(x, one)) <= 138 * Fraction(2) ** (b - 62) + Fraction(np.spacing(abs(got)) / 2)
+
+
+def _run(pmf, a, x0, lam, replicas, steps, uid_base=0, **kw):
+    run = inputs.RunSettings(**dict(dict(k=20.0, kT=1.0, dt=1e-3, gamma=1.0, n_steps=steps, n_equil=0, stride=50,
+                                         replicas=replicas, seed=21), **kw))
+    rr = pmf.pmf_run_windows(pmf.pmf_create_system_1d(a, x0), np.asarray(lam, dtype=np.float64),
+                             pmf.make_params(run, uid_base=uid_base))
+    return np.asarray(rr.final_state()[0]).reshape(len(lam), replicas)
+
+
+@pytest.mark.parametrize("a,lam", [(0.0, [-5.0, 0.0, 0.3, 2.0**20]), (2.0, [-1.5, 0.0, 1.2, 3.1, 30.0])])
+def test_bits_do_not_depend_on_the_other_windows(pmf, a, lam):
+    """Each window alone (same uids) and beside the others: the traps far away
+    neither widen its fixed-point range nor send it to FP64."""
+    together = _run(pmf, a, -0.4, lam, 3, 700)
+    for w, l in enumerate(lam):
+        assert np.array_equal(_run(pmf, a, -0.4, [l], 3, 700, uid_base=3 * w)[0], together[w]), l

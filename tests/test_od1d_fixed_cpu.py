@@ -1,5 +1,6 @@
 """The 1D integrator's fixed-point arithmetic on the host (the functions that
-the kernel compiles, no GPU): the guard of its range, and its rounding."""
+the kernel compiles, no GPU): the guard of its range, its rounding, and the
+choice of the range."""
 import math
 import os
 import shutil
@@ -84,3 +85,32 @@ def test_steps_round_to_either_side(a, k, dt, b):
         err += float(e)
         x0 = x1
     assert abs(err / N) <= 5 * math.sqrt(1.4 / N) + 0.5 * abs(X.astype(float).mean()) / 2.0**62 + 2 / 256
+
+
+def test_range_holds_the_motion_and_keeps_fp64s_precision():
+    """Over many models and traps: the range holds what it must, no step from
+    inside can wrap, and its unit stays below FP64's rounding of |x|, 2^b <= 128 |x| (the
+    error of a step is 1.2 units of 2^(b-62), FP64's |x| 2^-53.7)."""
+    g = np.random.default_rng(12)
+    taken = 0
+    for _ in range(20000):
+        a = float(g.choice([0.0, 2.0, 10 ** g.uniform(-6, 2), -(10 ** g.uniform(-3, 0))]))
+        x0, k, kT = float(g.normal(0, 1)), 10 ** g.uniform(-3, 8), 10 ** g.uniform(-4, 2)
+        dt = float(10 ** g.uniform(-6, 0) / (k + 8 * abs(a)))
+        far = float(abs(g.normal()) * 10 ** g.uniform(-2, 9))
+        near = float(far * g.choice([0.0, 1.0, g.random()]))
+        b = pmf.pmf_od1d_range(a, x0, k, kT, dt, 1.0, far, near)
+        if b is None:
+            continue
+        taken += 1
+        s, amp = math.sqrt(kT / k), math.sqrt(2 * kT * dt)
+        assert 2.0**b >= max(far, abs(x0), a != 0) + 6 * s
+        size = max(math.sqrt(kT / (k + 4 * abs(a))), near if a == 0 else min(near, 1.0) if a > 0 else 0.0)
+        assert 2.0**b <= 128 * size
+        assert abs(4 * a - k) * dt + abs(4 * a * dt) * 4.0**b + (6.8 * amp + k * dt * far) / 2.0**b < 1.0
+    assert taken > 2000
+
+
+@pytest.mark.parametrize("far,b", [(1.5, 2), (0.0, 2), (2.6, 2), (2.8, 3), (100.0, None)])
+def test_range_of_the_double_well(far, b):
+    assert pmf.pmf_od1d_range(2.0, -1.0, 20.0, 1.0, 1e-3, 1.0, far, far) == b
