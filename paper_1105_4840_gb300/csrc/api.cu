@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <memory>
 #include <string>
@@ -318,7 +319,7 @@ static pmf_status prepare_items(pmf_system *sys, const pmf_batch_item *items, in
         ri.w0 = w0;
         ri.nw = items[it].n_windows;
         ri.state_stride =
-            sys->model == PMF_MODEL_CHAIN ? sys->chains[ri.chain]->state_bytes_per_replica() : 2 * sizeof(double);
+            sys->model == PMF_MODEL_CHAIN ? sys->chains[ri.chain]->state_bytes_per_replica() : sizeof(Od1dState);
         ri.state_off = state_off;
         state_off += ri.state_stride * (size_t)(sequential ? 1 : ri.nw) * p->replicas;
         run->items.push_back(ri);
@@ -1590,7 +1591,7 @@ pmf_status pmf_run_adaptive(pmf_system *sys, const double *lambda0, int n0, cons
     const int N = chain ? sys->chains[p->chain]->n_beads() : 0;
     const int Np = chain ? sys->chains[p->chain]->n_padded() : 0;
     const bool fp64 = chain && sys->chains[p->chain]->precision() == PMF_FP64;
-    const size_t state_stride = chain ? sys->chains[p->chain]->state_bytes_per_replica() : 2 * sizeof(double);
+    const size_t state_stride = chain ? sys->chains[p->chain]->state_bytes_per_replica() : sizeof(Od1dState);
     for (int round = 0; round < ap->max_rounds; ++round) {
         std::sort(win.begin(), win.end(), [&](const Window &a, const Window &b) { return dir * a.lam < dir * b.lam; });
         Merged m;
@@ -2072,9 +2073,9 @@ pmf_status pmf_final_state(const pmf_run *run, double *pos, double *vel, size_t 
     if (run->sys->model == PMF_MODEL_1D_DOUBLEWELL) {
         if (n_written) *n_written = (size_t)n_rep;
         if (!pos || capacity < (size_t)n_rep) return fail(PMF_EINVAL, "pmf_final_state: capacity too small");
-        std::vector<double> st(2 * (size_t)n_rep);  // (x, pulling work) per simulation
-        CK(cudaMemcpy(st.data(), run->d_state, sizeof(double) * st.size(), cudaMemcpyDeviceToHost), "copy state");
-        for (int q = 0; q < n_rep; ++q) pos[q] = st[2 * (size_t)q];
+        // the positions alone, a field of the records
+        CK(cudaMemcpy2D(pos, sizeof(double), static_cast<const char *>(run->d_state) + offsetof(Od1dState, x), sizeof(Od1dState),
+                        sizeof(double), n_rep, cudaMemcpyDeviceToHost), "copy state");
         return PMF_OK;
     }
     size_t need = 0;

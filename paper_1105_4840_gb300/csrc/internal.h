@@ -146,7 +146,17 @@ struct Od1dParams {
     double a = 2.0, x0 = -1.0;
 };
 // Launches the noise pre-pass and the integration per block of noise_steps
-// steps; the state holds x and the pulling work per simulation (2 doubles).
+// steps; the state (an Od1dState per simulation) carries all a simulation is between blocks, without
+// rounding: how its steps are cut into blocks, which depends on the number of simulations in
+// the launch, leaves no trace in its bits.
+struct Od1dState {
+    double x;                  // position
+    long long fixed;           // the same in fixed point, or kNotFixed
+    double work;               // pulling work after the trap's first moves0 moves,
+    long long moves0, acc_h;   //   and the sum of the positions at its moves since
+    unsigned long long acc_l;
+};
+constexpr long long kNotFixed = (long long)0x8000000000000000ull;
 cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cudaStream_t st);
 long long od1d_noise_steps(int n_rep);
 struct RangeRule;

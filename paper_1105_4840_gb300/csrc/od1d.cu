@@ -22,7 +22,7 @@
 // (k dt/gamma) where no well contracts the map faster (a = 0, k = 1, dt = 1e-3,
 // b = 4: 7.5e-15 against FP64's 1.2e-15), so its mean is added to the terms
 // that are there anyway, cB - 1 and q_n (the same case: 6e-17).  A simulation that leaves |x| < 2^b
-// redoes the tile of steps it left in, and runs on, in FP64.
+// redoes the tile of steps it left in, and runs on, in FP64, until a tile ends within half the range.
 #include <algorithm>
 #include <cmath>
 
@@ -36,7 +36,7 @@ struct Od1dArgs {
     double x0, k;
     const double *lambda;
     const long long *nsteps_w, *nequil_w, *off_w, *tw;
-    double *state;              // [n_rep][2]: x and the accumulated pulling work
+    Od1dState *state;           // [n_rep]
     const double *start;
     float *xout;
     int *err;
@@ -118,7 +118,7 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
 // its loop took 403.  21 x 8 simulations x 2e4 steps, whole run with estimates:
 // 4.62 -> 1.80 ms; 256 pulled simulations x 4400 steps: 2.27 -> 0.75 ms.
 constexpr int kTile = 40;  // 41.5 KB of shared memory a CTA; 32 steps: 2.17 against 1.90 ms
-static_assert(kTile % 8 == 0, "unrolled by 8");
+static_assert(kTile % 8 == 0, "unrolled by 8; a Philox block is four steps");
 constexpr int kOd1dThreads = 128;
 
 // Two tiles' buffers in shared memory.
@@ -164,13 +164,11 @@ __device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTil
     double x = 0.0;
     bool dbl = true;
     if (m.live) {
-        x = a.c0 == 0 ? (a.start ? a.start[m.rep] : a.x0) : a.state[2 * m.rep];
+        x = a.c0 == 0 ? (a.start ? a.start[m.rep] : a.x0) : a.state[m.rep].x;
         if (m.fixed) {
             f = step_of(cA, a.cB1, m.range);
-            if (fabs(x) < scaled(1.0, m.range)) {
-                Xi = __double2ll_rn(x * m.scale);
-                dbl = false;
-            }
+            Xi = a.c0 == 0 ? (fabs(x) < scaled(1.0, m.range) ? __double2ll_rn(x * m.scale) : kNotFixed) : a.state[m.rep].fixed;
+            dbl = Xi == kNotFixed;
         }
     }
     for (long long i = 0; i < m.tiles; ++i) {
@@ -178,7 +176,7 @@ __device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTil
         const int b = (int)(i & 1);
         const int lim = m.end <= n0 ? 0 : (m.end - n0 < kTile ? (int)(m.end - n0) : kTile);
         const long long X0 = Xi;
-        bool redo = dbl && lim > 0;
+        bool redo = dbl && lim > 0, tile_dbl = dbl;
         if (!dbl) {
             sh.X[b][0][lane] = Xi;
             unsigned guard = 0;  // top bit: a position outside [-2^62, 2^62)
@@ -200,7 +198,7 @@ __device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTil
         }
         if (redo) {
             if (!dbl) x = (double)X0 * m.unit;
-            dbl = true;
+            dbl = tile_dbl = true;
             sh.X[b][0][lane] = __double_as_longlong(x);
 #pragma unroll 4
             for (int s = 0; s < lim; ++s) {
@@ -209,9 +207,13 @@ __device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTil
                 x = fma(x, fma(cA, x * x, cB), q);
                 sh.X[b][s + 1][lane] = __double_as_longlong(x);
             }
+            if (m.fixed && fabs(x) < scaled(0.5, m.range)) {  // well inside again
+                Xi = __double2ll_rn(x * m.scale);
+                dbl = false;
+            }
         }
         __syncwarp();
-        const unsigned mask = __ballot_sync(0xffffffffu, dbl);
+        const unsigned mask = __ballot_sync(0xffffffffu, tile_dbl);
         if (lane == 0) sh.dbl_mask[b] = mask;
         tile_barrier();
     }
@@ -219,8 +221,8 @@ __device__ __forceinline__ void integrate_tiles(const Od1dArgs &a, const Od1dTil
     if (!m.live || m.end <= a.c0) return;
     if (!dbl) x = (double)Xi * m.unit;
     if (!isfinite(x)) atomicOr(a.err, kErrNonFinite);
-    a.state[2 * m.rep] = x;
-    if (!a.wout) a.state[2 * m.rep + 1] = 0.0;
+    a.state[m.rep].x = x;
+    a.state[m.rep].fixed = dbl ? kNotFixed : Xi;
 }
 
 // Warps 1 - 3: the next tile's q_n, and the records of the finished one; no
@@ -250,9 +252,15 @@ __device__ __forceinline__ void record_tiles(const Od1dArgs &a, const Od1dTiles 
     if (m.live) {
         enter_window(a.sequential ? (int)(a.c0 / a.window_steps) : m.w, a.c0);
         if (a.wout) {
-            W = a.c0 == 0 ? 0.0 : a.state[2 * m.rep + 1];
             moves = a.c0 - 1 - a.nequil_w[0];
-            moves0 = moves = moves > 0 ? moves : 0;
+            moves = moves > 0 ? moves : 0;
+            if (a.c0 > 0) {
+                const Od1dState &st = a.state[m.rep];
+                W = st.work;
+                moves0 = st.moves0;
+                acc_h = st.acc_h;
+                acc_l = st.acc_l;
+            }
         }
     }
     // sum over the moves m of k vdt (lambda_1 + vdt (m - 1/2) - x)
@@ -309,7 +317,13 @@ __device__ __forceinline__ void record_tiles(const Od1dArgs &a, const Od1dTiles 
         if (i > 0) records(i - 1);
         tile_barrier();
     }
-    if (helper == 0 && a.wout && m.live && m.end > a.c0) a.state[2 * m.rep + 1] = moves != moves0 ? fixed_work() : W;
+    if (helper == 0 && a.wout && m.live && m.end > a.c0) {
+        Od1dState &st = a.state[m.rep];
+        st.work = W;
+        st.moves0 = moves0;
+        st.acc_h = acc_h;
+        st.acc_l = acc_l;
+    }
 }
 
 __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
@@ -340,10 +354,11 @@ __global__ void __launch_bounds__(kOd1dThreads) od1d_kernel(const Od1dArgs a)
 
 long long od1d_noise_steps(int n_rep)
 {
-    // at most 2^23 normals (64 MB) per launch, between 64 and 8192 steps
+    // at most 2^23 normals (64 MB) per launch, between 80 and 8160 steps, whole
+    // tiles: a tile begins at the same steps in every launch
     long long c = (1LL << 23) / (n_rep > 0 ? n_rep : 1);
-    c = c < 64 ? 64 : (c > 8192 ? 8192 : c);
-    return c & ~3LL;
+    c = c < 2 * kTile ? 2 * kTile : (c > 8192 ? 8192 : c);
+    return c - c % kTile;
 }
 
 // The range holds the trap, the start, the wells and six widths of the trap, and
@@ -368,7 +383,7 @@ RangeRule od1d_range_rule(const Od1dParams &m, double k, double kT, double dt, d
 
 cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cudaStream_t st)
 {
-    if (L.noise == nullptr || L.noise_steps < 4 || (L.noise_steps & 3) != 0 || (L.step_begin & 3) != 0)
+    if (L.noise == nullptr || L.noise_steps < kTile || L.noise_steps % kTile != 0 || L.step_begin % kTile != 0)
         return cudaErrorInvalidValue;
     if (L.sequential && L.window_steps < 1) return cudaErrorInvalidValue;
     Od1dArgs a{};
@@ -379,7 +394,7 @@ cudaError_t od1d_launch(const Od1dParams &m, const RunLaunch &L, int n_rep, cuda
     a.nequil_w = L.nequil_w;
     a.off_w = L.off_w;
     a.tw = L.tw;
-    a.state = reinterpret_cast<double *>(L.state);
+    a.state = reinterpret_cast<Od1dState *>(L.state);
     a.start = L.start;
     a.xout = L.xout;
     a.err = L.err;

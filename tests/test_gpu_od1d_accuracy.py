@@ -50,3 +50,33 @@ def test_bits_do_not_depend_on_the_other_windows(pmf, a, lam):
     together = _run(pmf, a, -0.4, lam, 3, 700)
     for w, l in enumerate(lam):
         assert np.array_equal(_run(pmf, a, -0.4, [l], 3, 700, uid_base=3 * w)[0], together[w]), l
+
+
+@pytest.mark.parametrize("start", [None, 5.5])
+def test_bits_do_not_depend_on_the_number_of_simulations(pmf, start):
+    """The same uids in launches of 2 and of 2100 simulations, whose steps come
+    in blocks of 8160 and 3960: from inside the range, and from outside (FP64
+    until it is back)."""
+    got = []
+    for replicas in (2, 2100):
+        run = inputs.RunSettings(k=20.0, kT=1.0, dt=1e-3, gamma=1.0, n_steps=8500, n_equil=3, stride=7, replicas=replicas, seed=9)
+        sysh, prm = pmf.pmf_create_system_1d(0.5, -1.0), pmf.make_params(run)
+        rr = (pmf.pmf_run_prepare(sysh, np.array([0.3]), prm) if start is None else
+              pmf.pmf_run_prepare_seeded(sysh, np.array([0.3]), prm, np.full(replicas, start)))
+        rr.launch()
+        rr.wait()
+        got.append((np.asarray(rr.final_state()[0])[:2], np.asarray(rr.x_samples()[0])[:2]))
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("dt", [1e-3, 0.02])
+def test_pulled_bits_do_not_depend_on_the_number_of_simulations(pmf, dt):
+    got = []
+    for replicas in (2, 2100):
+        run = inputs.RunSettings(k=20.0, kT=1.0, dt=dt, gamma=1.0, n_steps=8500, n_equil=30, stride=10, replicas=replicas, seed=9)
+        rr = pmf.pmf_run_prepare_smd(pmf.pmf_create_system_1d(2.0, -1.0), -1.2, 0.25e-3 / dt, pmf.make_params(run))
+        rr.launch()
+        rr.wait()
+        got.append((np.asarray(rr.final_state()[0])[:2], np.asarray(rr.x_samples()[0])[:2], np.asarray(rr.smd_work())[:2]))
+    for small, large in zip(*got):
+        assert np.array_equal(small, large)
