@@ -614,6 +614,10 @@ pmf_status pmf_run_adaptive(pmf_system *sys, const double *lambda0, int n0, cons
  * the run is in flight. */
 pmf_status pmf_run_set_queue_start(pmf_run *run, int64_t first_item);
 
+/* Test hook of pmf_free_energy_noalloc: leaves the counter in its fixed scratch at
+ * `value`, as calls that overlapped might.  The next call must not see it. */
+pmf_status pmf_noalloc_set_counter(uint32_t value);
+
 /* The integrator's Philox4x32-10 and Box-Muller on the GPU: blocks with
  * counters (c0 + i, c1, c2, c3), key (seed lo, seed hi), i < n_blocks.
  * raw[4 n_blocks] uint32 and normals[4 n_blocks] (FP32 as used by the FP32

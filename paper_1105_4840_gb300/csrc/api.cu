@@ -80,14 +80,12 @@ template <typename T> cudaError_t upload(T **d, const T *h, size_t n)
 }
 
 // Reduction scratch of `bytes` (reduce_scratch_bytes, or what is left of it
-// without the partials), its counter zeroed.
+// without the partials), and the counter in it.
 cudaError_t alloc_reduce(void **buf, size_t bytes, unsigned **counter)
 {
     cudaError_t e = cudaMalloc(buf, bytes);
-    if (e != cudaSuccess) return e;
-    const unsigned zero = 0;
-    *counter = reduce_counter(*buf, bytes);
-    return cudaMemcpy(*counter, &zero, sizeof(zero), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) *counter = reduce_counter(*buf, bytes);
+    return e;
 }
 
 }  // namespace
@@ -2063,6 +2061,13 @@ pmf_status pmf_free_energy_noalloc(const float *x, const double *lambda, int n_w
     if (!(k > 0) || !(kT > 0)) return fail(PMF_EINVAL, "pmf_free_energy_noalloc: need k > 0, kT > 0");
     cudaError_t e = reduce_noalloc_launch(x, lambda, n_windows, replicas, samples_per_window, k, kT, out, g_stream);
     if (e != cudaSuccess) return cuda_fail(e, "pmf_free_energy_noalloc");
+    return PMF_OK;
+}
+
+pmf_status pmf_noalloc_set_counter(uint32_t value)
+{
+    if (pmf_status s = need_device()) return s;
+    CK(noalloc_set_counter(value, g_stream), "pmf_noalloc_set_counter");
     return PMF_OK;
 }
 

@@ -190,7 +190,7 @@ struct ReduceLayout {
     const long long *off_w = nullptr;  // device [s]; null: windows of t_max samples a replica, end to end
     const long long *tw = nullptr;     // device [s]; null: t_max
     long long t_max = 0;               // most samples a replica of any window has
-    unsigned *counter = nullptr;       // device, 0 between launches: windows combined (see reduce_counter)
+    unsigned *counter = nullptr;       // device: windows combined (see reduce_counter); every call zeroes it
     int n_windows = 0, replicas = 0;
     double k = 0, kT = 1;
 };
@@ -202,7 +202,7 @@ enum ResultField {
 // scratch: device buffer of reduce_scratch_bytes(); out: device [kResFields][n_windows]
 size_t reduce_scratch_bytes(int n_windows, int replicas);
 // The counter at the end of a scratch buffer of `bytes` (reduce_scratch_bytes
-// or what is left of it after the partials); the allocation zeroes it.
+// or what is left of it after the partials).
 unsigned *reduce_counter(void *buffer, size_t bytes);
 cudaError_t reduce_launch(const ReduceLayout &L, void *scratch, double *out, cudaStream_t st);
 // The two halves of reduce_launch.  Per-replica partials, 5 doubles each,
@@ -222,6 +222,7 @@ cudaError_t combine_launch(const ReduceLayout &L, const void *partials, void *wi
 // per window, all pointers on the device.
 constexpr int kNoAllocMaxWindows = 1024;
 constexpr long long kNoAllocMaxWindowReplicas = 65536;  // n_windows * replicas
+cudaError_t noalloc_set_counter(unsigned value, cudaStream_t st);  // test hook
 cudaError_t reduce_noalloc_launch(const float *x, const double *lambda, int n_windows, int replicas,
                                   long long samples_per_window, double k, double kT, double *out, cudaStream_t st);
 // Eq. (5) / Eq. (15) after reduce_launch filled `scratch`: out[2 s + 1] =

@@ -290,6 +290,8 @@ __global__ void __launch_bounds__(kPartialThreads, G >= 4 ? 5 : 4) partial_kerne
     const long long T = samples_of(L, w), off = offset_of(L, w);
     const double li = L.lambda[w], ln = w + 1 < L.n_windows ? L.lambda[w + 1] : li;
     const float sgn = order_key(ln) < order_key(li) ? -1.f : 1.f;
+    // for the combination behind this grid, which touches it after this grid's end
+    if (L.counter != nullptr && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *L.counter = 0;
     if (threadIdx.x < 32) {
         tab_hi[threadIdx.x] = tab.hi[threadIdx.x];
         tab_lo[threadIdx.x] = tab.lo[threadIdx.x];
@@ -455,7 +457,7 @@ struct CombineArgs {
     const Partial *P;
     WindowOut *wo;
     double *out;
-    unsigned *counter;       // windows finished; 0 between launches (atomicInc wraps)
+    unsigned *counter;       // windows finished; set to 0 in every call before this grid starts
     double beta_h, beta_l;   // 1 / kT
     double k_beta, half_beta2;  // k / kT, 1 / (2 kT^2)
     double jk, inv_r;        // (R - 1) / R, 1 / R
@@ -715,7 +717,7 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) sh_last = atomicInc(A.counter, (unsigned)L.n_windows - 1) == (unsigned)L.n_windows - 1;
+    if (threadIdx.x == 0) sh_last = atomicAdd(A.counter, 1u) == (unsigned)L.n_windows - 1;
     __syncthreads();
     if (!sh_last) return;
     __threadfence();
@@ -905,6 +907,10 @@ cudaError_t combine_launch(const ReduceLayout &L, const void *P, void *window_sc
                            bool behind_partials)
 {
     if (L.counter == nullptr) return cudaErrorInvalidValue;
+    if (!behind_partials) {  // (the partials' grid zeroes it otherwise)
+        cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+    }
     CombineArgs A;
     A.P = static_cast<const Partial *>(P);
     A.wo = static_cast<WindowOut *>(window_scratch);
@@ -1031,9 +1037,9 @@ cudaError_t work_samples_launch(const ReduceLayout &L, int mode, long long sampl
 // cudaMalloc.  Every GPU that loads the library holds this array until the
 // process exits, and every call on that GPU reuses it: two calls whose work
 // overlaps on the GPU (different streams, or a second call before the first
-// has finished) write the same scratch and race.  Only the counter of
-// finished windows has to start at zero: it does when the module is loaded, and
-// every call leaves it so; each call rewrites every other entry it later reads.
+// has finished) write the same scratch and race.  Each call rewrites every entry
+// it later reads, the counter of finished windows too, so whatever an overlap
+// left there ends with the calls that overlapped.
 // ---------------------------------------------------------------------------
 
 namespace {
@@ -1103,6 +1109,16 @@ cudaError_t noalloc_scratch(void **out)
 }
 
 }  // namespace
+
+cudaError_t noalloc_set_counter(unsigned value, cudaStream_t st)
+{
+    void *base = nullptr;
+    cudaError_t e = noalloc_scratch(&base);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(reduce_counter(base, kNoAllocBytes), &value, sizeof(value), cudaMemcpyHostToDevice, st)) != cudaSuccess)
+        return e;
+    return cudaStreamSynchronize(st);
+}
 
 cudaError_t reduce_noalloc_launch(const float *x, const double *lambda, int n_windows, int replicas,
                                   long long samples_per_window, double k, double kT, double *out, cudaStream_t st)

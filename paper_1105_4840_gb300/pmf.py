@@ -149,6 +149,7 @@ def _load():
                                                      C.c_double, _D, _D, _D]
     L.pmf_free_energy_noalloc.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int64,
                                           C.c_double, C.c_double, C.c_void_p]
+    L.pmf_noalloc_set_counter.argtypes = [C.c_uint32]
     L.pmf_mlp_create.argtypes = [_F, C.c_double, C.c_double, C.POINTER(P)]
     L.pmf_mlp_destroy.argtypes = [P]
     L.pmf_mlp_destroy.restype = None
@@ -182,7 +183,7 @@ def _load():
                  "pmf_run_partials", "pmf_free_energy_from_partials", "pmf_work_distributions", "pmf_philox",
                  "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
-                 "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc",
+                 "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc", "pmf_noalloc_set_counter",
                  "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train",
                  "pmf_overlap", "pmf_run_adaptive", "pmf_chain_set_warps", "pmf_chain_set_grid", "pmf_chain_get_launch",
                  "pmf_chain_set_schedule", "pmf_chain_get_schedule", "pmf_chain_schedule_variant",
@@ -686,6 +687,11 @@ def pmf_run_adaptive(system: System, lambda0, params, mlp_init, threshold=0.3, m
                                trained=int(ta["trained"][q]), data_ovl=ta["data_ovl"][q, :max(nw - 1, 0)].copy()))
         meta["trace"] = rounds
     return meta, out
+
+
+def pmf_noalloc_set_counter(value):
+    """Test hook: the counter that calls which overlapped would leave."""
+    _check(lib.pmf_noalloc_set_counter(value), "pmf_noalloc_set_counter")
 
 
 def pmf_chain_set_warps(system: System, chain, warps):
