@@ -555,9 +555,15 @@ __device__ void profile(const ReduceLayout &L, const CombineArgs &A)
 // One CTA per window, in two halves that work side by side: warps 0 - 3 on the
 // exponential sums, 4 - 7 on the moments.  The compensated total of the
 // exponential sums comes from an exact split instead of a tree of TwoSums:
-// every e_r is cut at a common bit (adding and subtracting 1.5 2^K, 2^K >= 2 R
-// max e), the upper parts add up without rounding, the lower ones to
-// 2^-106 of the total.  The jackknife's sums are taken about the full estimate,
+// every e_r is cut at a common bit (adding and subtracting 1.5 2^K, 2 R max e <=
+// 2^K <= 8 R max e): the upper parts add up without rounding, the lower ones, at most
+// 2^(K-53) each, to within (R / 128 + 11) 4 R^2 2^-106 of the total (2^-90 at R =
+// 32, 2^-62 at 65536), below what a double shows of it.  Leaving out the largest
+// term may leave next to nothing, so its lower part is kept apart from the others'
+// sum: what is left then has a sum's own relative rounding however small it is, and for
+// every other r the rest holds the largest term.  (With the lower parts in one sum
+// a replica 61 kT above 31 others left 1e-5 wrong, one 75 kT above nothing at all.)
+// The jackknife's sums are taken about the full estimate,
 // which lies between the leave-one-out values, so one pass serves mean and
 // spread.  The last CTA to finish turns the windows into the profiles.
 template <bool SMEM>
@@ -566,7 +572,7 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
     extern __shared__ double E[];  // [replicas] when SMEM
     __shared__ long long red_key[2][kHalfWarps];
     __shared__ double red[2][kHalfWarps][3], red_q[2][kHalfWarps][2];
-    __shared__ double sh_log;
+    __shared__ double sh_log, sh_top[2];  // (the largest term's upper and lower part)
     __shared__ int sh_last;
     const int w = blockIdx.x, R = L.replicas, lane = threadIdx.x & 31;
     const int half = threadIdx.x >= kHalf, t = threadIdx.x - half * kHalf, hw = t >> 5;
@@ -574,6 +580,7 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
     cudaGridDependencySynchronize();  // the partials are there (returns at once after an ordinary launch)
     const bool active = hw * 32 < R;  // the other warps hold no replica and keep off the FP64 unit
     double m = 0.0;
+    int top = 0;  // the replica of the largest term (to 2^-20; half 0)
     // replica r's exponential sum brought to the window's common shift m
     auto e_of = [&](int r) {
         if (!(p[r].n > 0)) return 0.0;
@@ -601,9 +608,10 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
             const double e = e_of(r);
             if (r == t) e0 = e;
             if (SMEM) E[r] = e;
-            emax = max(emax, __double_as_longlong(e));
+            emax = max(emax, (__double_as_longlong(e) & ~0xffffffffLL) | r);
         }
         emax = half_max(emax, 1);
+        top = (int)(emax & 0xffffffffLL);
         if (active) {
             // 1.5 2^K with 2^K >= 2 R max e (NaN and overflowing terms end up in the sums either way)
             const int K = min(max((int)(emax >> 52) - 1023 + 2 + A.log2_r, -1022), 1023);
@@ -613,7 +621,12 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
                 const double e = r == t ? e0 : (SMEM ? E[r] : e_of(r));
                 const double u = (e + cut) - cut;
                 hi += u;
-                lo += e - u;
+                if (r == top) {
+                    sh_top[0] = u;
+                    sh_top[1] = e - u;
+                } else {
+                    lo += e - u;
+                }
             }
             const double v = warp_sum2(hi, lo, lane);
             if ((lane & 15) == 0) red[0][hw][lane >> 4] = v;
@@ -650,15 +663,18 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
     double q1 = 0, q2 = 0;  // jackknife: sums of the leave-one-out values minus the full estimate, and of their squares
     double lf = 0.0;
     if (half == 0) {
-        double Shi = 0, Slo = 0, n = 0;
+        double Shi = 0, Slo = 0, n = 0, th = 0, rest = 0;
         if (active || closing) {
-            const double th = total(0, 0), tl = total(0, 1);
+            th = total(0, 0);
+            rest = total(0, 1);
+            const double tl = rest + sh_top[1];
             n = total(1, 0);
             Shi = th + tl;
             Slo = tl - (Shi - th);
         }
         auto log_without = [&](int r) {
-            return log(sum_without(Shi, Slo, SMEM ? E[r] : e_of(r)) / (n - p[r].n));
+            const bool largest = r == top;  // (selects, not a branch: two FP64 operations either way)
+            return log(sum_without(largest ? th : Shi, largest ? rest : Slo, largest ? sh_top[0] : (SMEM ? E[r] : e_of(r))) / (n - p[r].n));
         };
         if (closing && lane == 0) sh_log = log((Shi + Slo) / n);  // beside the leave-one-out logarithms
         double l0 = 0.0;
