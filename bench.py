@@ -716,7 +716,7 @@ def bench_spp(args, pmf, torch, stream):
             "unit": "replica-steps/s", "ms_per_step": t, "steps": args.steps, "warmup": args.warmup,
             "config": {"simulations": run.replicas, "windows": int(run.lambdas.size),
                        "md_steps_per_window": run.n_steps, "warps_per_replica": warps,
-                       "launch": f"persistent, {'auto' if ctas == 0 else ctas} CTAs, segments <= {seg} steps"},
+                       "launch": f"persistent, {'auto' if ctas == 0 else ctas} CTAs, segments <= {seg or 1000} steps"},
             "clocks": {"sm_mhz": clk.get("sm_mhz"), "sm_max_mhz": clk.get("sm_max_mhz"),
                        "reasons": clk.get("reasons")},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -1107,7 +1107,7 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": workload_config(run, world),
             "launch": {"warps_per_replica": warps, "ctas": "auto" if grid_ctas == 0 else grid_ctas,
-                       "segment_steps": seg_steps, "mode": "persistent",
+                       "segment_steps": seg_steps or "auto", "mode": "persistent",
                        "schedule_variant": pmf.pmf_chain_get_schedule(sysh, 0)},
             "e2e": {"value": e2e_value, "unit": "replica-steps/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h},

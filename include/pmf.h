@@ -440,7 +440,7 @@ pmf_status pmf_chain_set_warps(pmf_system *sys, int chain, int warps);
  * no SM idles when the replica count is not a multiple of the SM count.
  * Trajectories are bit-identical for every shape (the state record holds
  * the whole integrator state between segments).  Default: ctas = 0,
- * seg_steps = 1000.  Batched runs always use one CTA per replica. */
+ * seg_steps = 0.  Batched runs always use one CTA per replica. */
 pmf_status pmf_chain_set_grid(pmf_system *sys, int chain, int ctas, int seg_steps);
 /* Schedule cost model of chain `chain` (see pmf_chain_schedule_variant; the
  * work schedule is rebuilt, results are bit-reproducible for a given
@@ -448,7 +448,9 @@ pmf_status pmf_chain_set_grid(pmf_system *sys, int chain, int ctas, int seg_step
 pmf_status pmf_chain_set_schedule(pmf_system *sys, int chain, int variant);
 pmf_status pmf_chain_get_schedule(const pmf_system *sys, int chain, int *variant);
 /* The current warps per replica, ctas and seg_steps of chain `chain` (as set
- * by the calls above or chosen by pmf_chain_autotune); NULL outputs skipped. */
+ * by the calls above or chosen by pmf_chain_autotune, 0 where the choice was left to
+ * the library): handed to pmf_chain_set_grid they give the same launches.  NULL
+ * outputs skipped. */
 pmf_status pmf_chain_get_launch(const pmf_system *sys, int chain, int *warps, int *ctas, int *seg_steps);
 /* Time probe_steps steps of the given run (every window and replica, one
  * warm-up launch and the best of two timed launches each; use several

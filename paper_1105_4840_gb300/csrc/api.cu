@@ -1879,7 +1879,7 @@ pmf_status pmf_chain_get_launch(const pmf_system *sys, int chain, int *warps, in
     const ChainModel &m = *sys->chains[chain];
     if (warps) *warps = m.warps();
     if (ctas) *ctas = m.grid_ctas();
-    if (seg_steps) *seg_steps = m.seg_steps();
+    if (seg_steps) *seg_steps = m.seg_request();
     return PMF_OK;
 }
 

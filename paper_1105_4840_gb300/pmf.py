@@ -703,7 +703,8 @@ def pmf_chain_set_grid(system: System, chain, ctas, seg_steps=0):
 
 
 def pmf_chain_get_launch(system: System, chain=0):
-    """(warps, ctas, seg_steps) of a chain's launch shape."""
+    """(warps, ctas, seg_steps) of a chain's launch shape as it was set; 0 ctas
+    or steps: left to the library."""
     w, c, g = C.c_int(), C.c_int(), C.c_int()
     _check(lib.pmf_chain_get_launch(system.handle, chain, C.byref(w), C.byref(c), C.byref(g)), "pmf_chain_get_launch")
     return w.value, c.value, g.value
