@@ -653,6 +653,12 @@ pmf_status pmf_od1d_range(double a, double x0, double k, double kT, double dt, d
 pmf_status pmf_od1d_fixed_map(double cA, double cB1, int range_log2, int64_t X0, int n, const int64_t *q, int64_t *X,
                               int *outside);
 
+/* The surrogate's SiLU and its slope, computed without divisions, against the
+ * divisions as written, for the `count` floats (a multiple of 16, up to 2^32) whose bits
+ * begin at `first`: *differing receives how many results differ (zeros of either
+ * sign and NaNs are alike). */
+pmf_status pmf_mlp_silu_check(uint32_t first, uint64_t count, uint64_t *differing);
+
 /* Overlap coefficients ovl[i] = int min(p_i, p_{i+1}) dx, i < n - 1, of the
  * Gaussians N(mu_i, exp(log_var_i)) (host arrays), computed by the kernel
  * the adaptive protocol uses. */

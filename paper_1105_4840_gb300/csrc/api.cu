@@ -1420,6 +1420,22 @@ pmf_status pmf_mlp_gradient(pmf_mlp *mlp, const double *lambda, const float *x, 
     return PMF_OK;
 }
 
+pmf_status pmf_mlp_silu_check(uint32_t first, uint64_t count, uint64_t *differing)
+{
+    if (!differing || count % 16 != 0 || count > (1ULL << 32)) return fail(PMF_EINVAL, "pmf_mlp_silu_check: bad argument");
+    if (pmf_status s = need_device()) return s;
+    *differing = 0;
+    if (count == 0) return PMF_OK;
+    unsigned long long *d = nullptr, h = 0;
+    CK(upload(&d, &h, 1), "pmf_mlp_silu_check");
+    std::unique_ptr<unsigned long long, cudaError_t (*)(void *)> guard(d, cudaFree);
+    CK(mlp_silu_check_launch(first, count / 16, d, g_stream), "pmf_mlp_silu_check");
+    CK(cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, g_stream), "copy");
+    CK(cudaStreamSynchronize(g_stream), "sync");
+    *differing = h;
+    return PMF_OK;
+}
+
 pmf_status pmf_mlp_set_split(pmf_mlp *mlp, int split)
 {
     if (!mlp || (split != 0 && split != 1)) return fail(PMF_EINVAL, "pmf_mlp_set_split: bad argument");

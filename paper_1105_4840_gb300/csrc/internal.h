@@ -263,6 +263,8 @@ struct MlpLaunch {
     int tile_cap = 0;
 };
 cudaError_t mlp_launch(const MlpLaunch &L, cudaStream_t st);
+// differing += how many of 2 x 16 x groups activations and slopes differ (silu_check_kernel)
+cudaError_t mlp_silu_check_launch(uint32_t first, unsigned long long groups, unsigned long long *differing, cudaStream_t st);
 
 // Learned window placement (adaptive.cu)
 cudaError_t overlap_launch(const double *mu, const double *log_var, int n, double *ovl, cudaStream_t st);

@@ -157,6 +157,7 @@ def _load():
     L.pmf_mlp_predict.argtypes = [P, _D, C.c_int, _D, _D]
     L.pmf_mlp_gradient.argtypes = [P, _D, _F, C.c_int, _F, _D]
     L.pmf_mlp_train.argtypes = [P, P, C.c_int, C.c_int, C.c_double, C.c_uint64, _D]
+    L.pmf_mlp_silu_check.argtypes = [C.c_uint32, C.c_uint64, C.POINTER(C.c_uint64)]
     L.pmf_mlp_set_split.argtypes = [P, C.c_int]
     L.pmf_overlap.argtypes = [_D, _D, C.c_int, _D]
     L.pmf_run_adaptive.argtypes = [P, _D, C.c_int, C.POINTER(RunParams), C.POINTER(AdaptiveParams),
@@ -184,7 +185,7 @@ def _load():
                  "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
                  "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc", "pmf_noalloc_set_counter",
-                 "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train",
+                 "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train", "pmf_mlp_silu_check",
                  "pmf_overlap", "pmf_run_adaptive", "pmf_chain_set_warps", "pmf_chain_set_grid", "pmf_chain_get_launch",
                  "pmf_chain_set_schedule", "pmf_chain_get_schedule", "pmf_chain_schedule_variant",
                  "pmf_chain_autotune", "pmf_fp32_peak", "pmf_fp64_peak", "pmf_set_stream"):
@@ -632,6 +633,14 @@ class Mlp:
         loss = C.c_double()
         _check(lib.pmf_mlp_train(self.handle, run.handle, steps, batch, lr, seed, C.byref(loss)), "pmf_mlp_train")
         return loss.value
+
+
+def pmf_mlp_silu_check(first, count):
+    """How many of the surrogate's activations and slopes differ from those by
+    divisions, over the `count` floats whose bits begin at `first`."""
+    n = C.c_uint64()
+    _check(lib.pmf_mlp_silu_check(first, count, C.byref(n)), "pmf_mlp_silu_check")
+    return n.value
 
 
 def pmf_overlap(mu, log_var):
