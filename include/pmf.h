@@ -659,6 +659,10 @@ pmf_status pmf_od1d_fixed_map(double cA, double cB1, int range_log2, int64_t X0,
  * sign and NaNs are alike). */
 pmf_status pmf_mlp_silu_check(uint32_t first, uint64_t count, uint64_t *differing);
 
+/* Test hook of pmf_mlp_train: cluster = 0 trains this surrogate by launches per step
+ * with 2 to 8 tiles too (1, the default: as one cluster).  The same bits. */
+pmf_status pmf_mlp_set_cluster(pmf_mlp *mlp, int cluster);
+
 /* Overlap coefficients ovl[i] = int min(p_i, p_{i+1}) dx, i < n - 1, of the
  * Gaussians N(mu_i, exp(log_var_i)) (host arrays), computed by the kernel
  * the adaptive protocol uses. */

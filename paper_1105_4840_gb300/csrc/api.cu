@@ -1291,6 +1291,7 @@ struct pmf_mlp {
     int t = 0;
     double c = 0, h = 1;
     int split = 1;                   // training: one CTA per 128-sample tile
+    bool cluster = true;             //   up to 8 of them as a cluster (off in tests only)
     float *tile_grad = nullptr;      // [tile_cap][kMlpParams]
     double *tile_loss = nullptr;     // [tile_cap]
     int tile_cap = 0;
@@ -1358,6 +1359,7 @@ static pmf_status mlp_run(pmf_mlp *mlp, MlpLaunch &L, const char *where)
             mlp->tile_cap = tiles;
         }
         L.split = true;
+        L.cluster = mlp->cluster;
         L.tile_grad = mlp->tile_grad;
         L.tile_loss = mlp->tile_loss;
         L.tile_cap = mlp->tile_cap;
@@ -1440,6 +1442,13 @@ pmf_status pmf_mlp_set_split(pmf_mlp *mlp, int split)
 {
     if (!mlp || (split != 0 && split != 1)) return fail(PMF_EINVAL, "pmf_mlp_set_split: bad argument");
     mlp->split = split;
+    return PMF_OK;
+}
+
+pmf_status pmf_mlp_set_cluster(pmf_mlp *mlp, int cluster)
+{
+    if (!mlp || (cluster != 0 && cluster != 1)) return fail(PMF_EINVAL, "pmf_mlp_set_cluster: bad argument");
+    mlp->cluster = cluster != 0;
     return PMF_OK;
 }
 

@@ -258,6 +258,7 @@ struct MlpLaunch {
     // tile_grad [tile_cap][kMlpParams] and tile_loss [tile_cap] are the caller's
     // scratch for the latter
     bool split = false;
+    bool cluster = true;  // off (tests only): launches per step with 2 to 8 tiles too
     float *tile_grad = nullptr;
     double *tile_loss = nullptr;
     int tile_cap = 0;

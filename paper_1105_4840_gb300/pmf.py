@@ -159,6 +159,7 @@ def _load():
     L.pmf_mlp_train.argtypes = [P, P, C.c_int, C.c_int, C.c_double, C.c_uint64, _D]
     L.pmf_mlp_silu_check.argtypes = [C.c_uint32, C.c_uint64, C.POINTER(C.c_uint64)]
     L.pmf_mlp_set_split.argtypes = [P, C.c_int]
+    L.pmf_mlp_set_cluster.argtypes = [P, C.c_int]
     L.pmf_overlap.argtypes = [_D, _D, C.c_int, _D]
     L.pmf_run_adaptive.argtypes = [P, _D, C.c_int, C.POINTER(RunParams), C.POINTER(AdaptiveParams),
                                    C.POINTER(AdaptiveInfo), C.POINTER(FreeEnergyResult)]
@@ -185,7 +186,7 @@ def _load():
                  "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
                  "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc", "pmf_noalloc_set_counter",
-                 "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train", "pmf_mlp_silu_check",
+                 "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train", "pmf_mlp_silu_check", "pmf_mlp_set_cluster",
                  "pmf_overlap", "pmf_run_adaptive", "pmf_chain_set_warps", "pmf_chain_set_grid", "pmf_chain_get_launch",
                  "pmf_chain_set_schedule", "pmf_chain_get_schedule", "pmf_chain_schedule_variant",
                  "pmf_chain_autotune", "pmf_fp32_peak", "pmf_fp64_peak", "pmf_set_stream"):
@@ -628,6 +629,10 @@ class Mlp:
 
     def set_split(self, split):
         _check(lib.pmf_mlp_set_split(self.handle, int(split)), "pmf_mlp_set_split")
+
+    def set_cluster(self, cluster):
+        """Test hook: False trains by launches per step at every tile count."""
+        _check(lib.pmf_mlp_set_cluster(self.handle, int(cluster)), "pmf_mlp_set_cluster")
 
     def train(self, run, steps, batch, lr, seed):
         loss = C.c_double()
