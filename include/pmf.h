@@ -633,6 +633,9 @@ pmf_status pmf_philox(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint
 pmf_status pmf_chain_forces(pmf_system *sys, int chain, const double *pos, double lambda,
                             double k, double *forces);
 
+/* 1 / sqrt(v[i]) as the FP64 chains' pair forces compute it (host arrays). */
+pmf_status pmf_rsqrt(const double *v, int n, double *out);
+
 /* The records that one of the 1D integrator's three helper warps takes in a
  * window of n_equil equilibration steps, from step `from` on (host, no GPU
  * needed): record number at[i] is taken at the end of step step[i], i < n.

@@ -2154,6 +2154,23 @@ pmf_status pmf_philox(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2, uint
     return PMF_OK;
 }
 
+pmf_status pmf_rsqrt(const double *v, int n, double *out)
+{
+    if (n < 0 || (n > 0 && (!v || !out))) return fail(PMF_EINVAL, "pmf_rsqrt: bad argument");
+    if (pmf_status s = need_device()) return s;
+    if (n == 0) return PMF_OK;
+    struct Tmp {
+        double *v = nullptr, *out = nullptr;
+        ~Tmp() { cudaFree(v); cudaFree(out); }
+    } t;
+    CK(upload(&t.v, v, n), "pmf_rsqrt");
+    CK(cudaMalloc(&t.out, sizeof(double) * n), "pmf_rsqrt");
+    CK(rsqrt_launch(t.v, n, t.out, g_stream), "pmf_rsqrt");
+    CK(cudaMemcpyAsync(out, t.out, sizeof(double) * n, cudaMemcpyDeviceToHost, g_stream), "copy");
+    CK(cudaStreamSynchronize(g_stream), "sync");
+    return PMF_OK;
+}
+
 pmf_status pmf_od1d_records(int helper, int64_t n_equil, int stride, int64_t from, int n, int64_t *at, int64_t *step)
 {
     if (helper < 0 || helper >= kOd1dHelpers || n_equil < 0 || stride < 1 || from < 0 || n < 0 || (n > 0 && (!at || !step)))

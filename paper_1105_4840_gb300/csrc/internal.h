@@ -145,6 +145,8 @@ size_t pack_plan_smem(const PackPlan *plan);
 struct Od1dParams {
     double a = 2.0, x0 = -1.0;
 };
+// out[i] = the FP64 pairs' 1 / sqrt(v[i]) (device arrays)
+cudaError_t rsqrt_launch(const double *v, int n, double *out, cudaStream_t st);
 // Launches the noise pre-pass and the integration per block of noise_steps
 // steps; the state (an Od1dState per simulation) carries all a simulation is between blocks, without
 // rounding: how its steps are cut into blocks, which depends on the number of simulations in

@@ -135,6 +135,7 @@ def _load():
     L.pmf_chain_forces.argtypes = [P, C.c_int, _D, C.c_double, C.c_double, _D]
     L.pmf_chain_schedule.argtypes = [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int), C.c_size_t,
                                      C.POINTER(C.c_size_t), C.POINTER(C.c_int)]
+    L.pmf_rsqrt.argtypes = [_D, C.c_int, _D]
     L.pmf_od1d_records.argtypes = [C.c_int, C.c_int64, C.c_int, C.c_int64, C.c_int, _I64, _I64]
     L.pmf_od1d_range.argtypes = [C.c_double] * 8 + [C.POINTER(C.c_int)]
     L.pmf_od1d_fixed_map.argtypes = [C.c_double, C.c_double, C.c_int, C.c_int64, C.c_int, _I64, _I64, C.POINTER(C.c_int)]
@@ -183,7 +184,7 @@ def _load():
                  "pmf_run_wait", "pmf_get_run_info", "pmf_x_samples", "pmf_work_samples",
                  "pmf_free_energy", "pmf_free_energy_from_samples", "pmf_final_state",
                  "pmf_run_partials", "pmf_free_energy_from_partials", "pmf_work_distributions", "pmf_philox",
-                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
+                 "pmf_chain_forces", "pmf_chain_schedule", "pmf_rsqrt", "pmf_od1d_records", "pmf_od1d_fixed_map", "pmf_od1d_range", "pmf_run_reduce", "pmf_run_set_queue_start", "pmf_run_set_batch_launch",
                  "pmf_run_get_batch_launch", "pmf_run_batch_autotune", "pmf_state_free_energy",
                  "pmf_state_free_energy_from_samples", "pmf_free_energy_noalloc", "pmf_noalloc_set_counter",
                  "pmf_mlp_create", "pmf_mlp_get_params", "pmf_mlp_predict", "pmf_mlp_gradient", "pmf_mlp_train", "pmf_mlp_silu_check", "pmf_mlp_set_cluster",
@@ -722,6 +723,14 @@ def pmf_chain_get_launch(system: System, chain=0):
     w, c, g = C.c_int(), C.c_int(), C.c_int()
     _check(lib.pmf_chain_get_launch(system.handle, chain, C.byref(w), C.byref(c), C.byref(g)), "pmf_chain_get_launch")
     return w.value, c.value, g.value
+
+
+def pmf_rsqrt(v):
+    """1 / sqrt(v) as the FP64 chains' pair forces compute it."""
+    v = np.ascontiguousarray(v, dtype=np.float64)
+    out = np.zeros_like(v)
+    _check(lib.pmf_rsqrt(_dp(v), v.size, _dp(out)), "pmf_rsqrt")
+    return out
 
 
 def pmf_od1d_records(helper, n_equil, stride, start, n):
