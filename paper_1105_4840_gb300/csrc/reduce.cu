@@ -673,8 +673,10 @@ __global__ void __launch_bounds__(kWindowThreads) combine_kernel(const ReduceLay
             Slo = tl - (Shi - th);
         }
         auto log_without = [&](int r) {
-            const bool largest = r == top;  // (selects, not a branch: two FP64 operations either way)
-            return log(sum_without(largest ? th : Shi, largest ? rest : Slo, largest ? sh_top[0] : (SMEM ? E[r] : e_of(r))) / (n - p[r].n));
+            const double e = SMEM ? E[r] : e_of(r);
+            // (from half the total on; selects, not a branch: two FP64 operations either way)
+            const bool most = r == top && __double2hiint(Shi) - __double2hiint(e) < 1 << 20;
+            return log(sum_without(most ? th : Shi, most ? rest : Slo, most ? sh_top[0] : e) / (n - p[r].n));
         };
         if (closing && lane == 0) sh_log = log((Shi + Slo) / n);  // beside the leave-one-out logarithms
         double l0 = 0.0;
