@@ -356,8 +356,10 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return f2
 // overlap the steps.  What bounds a piece is the number of registers for that
 // overlap: alone on its scheduler a warp takes about 230 cycles per ring step
 // with 128 registers, 300 with 96, against 100 of FP32 pipe; SCALAR (both FMAs
-// of the pair as scalar FFMAs) is the faster form with 128 registers and
-// spills with 96.  Same results in both forms.  One CTA per SM, 4 warps:
+// of the pair as scalar FFMAs) is the faster form in the build of four warps with 128
+// registers, the only one that uses it, and spills with 96; in the helper, eight-warp
+// and packed builds, which have 128 to 168, it was not compared.  Same results in
+// both forms.  One CTA per SM, 4 warps:
 // 104 beads 7890 -> 7170 cycles a step, 333 beads 41150 -> 31480; 672 replicas
 // of 104 beads 100.4 -> 107.0 M replica-steps/s (1000 steps).
 //
@@ -1026,8 +1028,9 @@ template <typename R, int NW, int NH, int CTAS, bool SMD>
 __global__ void __launch_bounds__((NW + NH) * 32, CTAS) chain_kernel(const ChainArgs<R> a)
 // SMD: the constant-velocity pulling variant (a separate instantiation, so
 // the window runs carry none of its per-step work bookkeeping).
-// FP32 with 4 warps: five CTAs per SM fit; 6 and 8 warps trade occupancy for
-// registers.  Two modes:
+// CTAS per SM (launch bounds) sets the registers: 4 warps four CTAs (128) or, for
+// short chains, five (96); 5, 6 and 8 warps four, three and two; helpers one or
+// two (see ChainModel::launch).  Two modes:
 //  * one CTA per replica (blockIdx.x), steps [step_begin, step_end);
 //  * persistent: gridDim.x CTAs take (segment, replica) items of seg_steps
 //    steps from a global queue, so replicas migrate between CTAs and every SM

@@ -113,10 +113,10 @@ __global__ void od1d_noise_kernel(const Od1dArgs a, long long *q)
 // next tile's q_n and turn the previous tile's positions into samples and
 // pulling work, so the dependent chain carries nothing else.  What bounds it is
 // that chain: 118 cycles a step by itself (a product of limbs is four dependent
-// 32 x 32 -> 64 multiplies of 9 - 12 cycles and a split), about 145 with the
+// 32 x 32 -> 64 multiplies of 9 - 12 cycles and a split), about 130 with the
 // tile's barrier; one thread per simulation in FP64 with loads and samples in
 // its loop took 403.  21 x 8 simulations x 2e4 steps, whole run with estimates:
-// 4.62 -> 1.80 ms; 256 pulled simulations x 4400 steps: 2.27 -> 0.75 ms.
+// 4.61 -> 1.72 ms; 256 pulled simulations x 4400 steps: 2.24 -> 0.68 ms.
 constexpr int kTile = 40;  // 41.5 KB of shared memory a CTA; 32 steps: 2.17 against 1.90 ms
 static_assert(kTile % 8 == 0, "unrolled by 8; a Philox block is four steps");
 constexpr int kOd1dThreads = 128;

@@ -20,8 +20,9 @@
 // FP64 operations (64 cycles each for one warp of this GPU), so stages 2 and 3
 // spend as few of them in sequence as they can and run independent ones on
 // different warps.  21 windows x 32 replicas x 3600 samples, back to back:
-// four launches (layout, partials, windows, profiles) 65.6 us, now 30.7 us;
-// 5 x 4 x 256: 49.2 us, now 20.5 us; 64 x 512 x 1801: 724 us, now 274 us.
+// four launches (layout, partials, windows, profiles) 65.6 us, now 28.7 us;
+// 5 x 4 x 256: 49.2 us, now 16.4 to 18.4 us from one call of the measurement to
+// the next; 64 x 512 x 1801: 724 us, now 272 us.
 #include <math.h>
 #include <stddef.h>
 
@@ -902,7 +903,7 @@ cudaError_t partials_launch(const ReduceLayout &L, void *P, cudaStream_t st)
 
 // behind_partials: the stream's last operation is this call's partials launch,
 // whose tail the combination's launch overlaps (it waits for that grid before it
-// reads): 5 x 4 x 256 samples 20.5 -> 17.3 us, 21 x 32 x 3600 30.7 -> 28.7 us.
+// reads): 5 x 4 x 256 samples 20.5 -> 17.3 us (first measured; see the top of the file), 21 x 32 x 3600 30.7 -> 28.7 us.
 // Behind anything else (gathered partials) an ordinary launch.
 template <typename K>
 static cudaError_t launch_combine(K kernel, size_t smem, bool behind_partials, cudaStream_t st, const ReduceLayout &L,
