@@ -134,7 +134,13 @@ struct Od1dSim {
     long long end, tiles;     // its last step (its window's step count), the launch's tiles
     double scale, unit;       // 2^S and 2^-S
 };
-__device__ __forceinline__ void tile_barrier() { asm volatile("bar.sync 0, %0;" ::"n"(kOd1dThreads) : "memory"); }
+// All four warps, from either role's loop.  The lanes of a warp, which run loops of
+// their own lengths, come together first: the barrier wants whole warps.
+__device__ __forceinline__ void tile_barrier()
+{
+    __syncwarp();
+    asm volatile("bar.sync 0, %0;" ::"n"(kOd1dThreads) : "memory");
+}
 // Rows row, row + STEP, ... of tile i: all loads, then all stores.  A load and its
 // store at a time are 14 latencies a helper, longer than the integrating
 // warp's 40 steps (21 x 8 x 2e4 steps: 2350 us, now 1712).
